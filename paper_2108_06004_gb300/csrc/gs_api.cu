@@ -1,12 +1,15 @@
 // C ABI of the gs-SGD compression library: argument validation, the sketch object, hash
 // coefficient derivation, and composition of the kernels into the calls of gs_sketch.h.
+#include <algorithm>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <string>
 #include <unordered_map>
 #include <vector>
 
+#include "chain_plan.h"
 #include "gs_common.cuh"
 
 struct gs_sketch {
@@ -17,6 +20,8 @@ struct gs_sketch {
   float* tables;  // groups * r*c*W
   float* merged;  // r*c
   int device;
+  // c a power of two: the convergents of every row's rotation (chain_plan.h), else empty
+  std::vector<std::vector<gs::Convergent>> rotation;
 };
 
 // Events recorded between the phases of a step while it is captured into a plan, where each
@@ -92,6 +97,14 @@ void derive_coefficients(int r, uint64_t seed, gs::HashCoeffs& h) {
 // and 96 MB thrashes; 8-wide groups with one 64 MB row per pass beat 4-wide groups.
 constexpr size_t kRowBudget = size_t(64) << 20;
 constexpr size_t kPassBudget = size_t(48) << 20;
+// Vectors up to this size stay in L2 from one row of a chained insert to the next.
+constexpr size_t kResidentBytes = size_t(64) << 20;
+// Shortest stride of a chain: 16 CTAs of chains, so that the last CTA's idle lanes stay few.
+constexpr int64_t kMinStride = 4096;
+// 8-wide groups insert directly from this length on.
+constexpr int64_t kDirectMinDim = int64_t(1) << 22;
+// Up to this many cell updates per worker every row is inserted directly.
+constexpr int64_t kFewUpdates = int64_t(1) << 20;
 
 // Widest group (up to 16, not wider than the worker count rounded up to a power of two) whose
 // single table row fits the row budget.  16-wide groups are used only when the whole group
@@ -168,9 +181,64 @@ gs_status check_vec(const void* p, const char* name) {
 
 cudaStream_t as_stream(gs_stream s) { return reinterpret_cast<cudaStream_t>(s); }
 
+// Inserts the vectors e[0..nw) of length d by chains into rows [j0, r) of the table whose cell
+// (row j, bucket b) is cells[(j * c + b) * pitch]; W: workers of a cell written.
+gs_status insert_chains(const gs_sketch* sk, float* cells, int pitch, int W, int j0, const float* const* e, int nw,
+                        int64_t d, cudaStream_t s) {
+  if (j0 >= sk->r) return GS_OK;
+  gs::ChainParams p;
+  std::memset(&p, 0, sizeof(p));
+  for (int w = 0; w < nw; ++w) p.e[w] = e[w];
+  p.d = d;
+  p.cmask = (uint32_t)sk->c - 1;
+  p.nw = nw;
+  p.pitch = pitch;
+  p.nrows = sk->r - j0;
+  p.resident = (size_t)d * nw * sizeof(float) <= kResidentBytes ? 1 : 0;
+  // Chains as long as two waves of 1536 threads per SM allow, and 32 at most: longer ones leave
+  // too few CTAs to even out the last wave (d = 25,557,032, 4 rows: 16, 32, 64 steps all within 1 %).
+  const int64_t lanes = (int64_t)gs::device_info().sms * 1536 * 2;
+  const int64_t max_steps = std::min<int64_t>(32, std::max<int64_t>(1, p.nrows * d / lanes));
+  for (int j = j0; j < sk->r; ++j) {
+    gs::ChainRow& row = p.row[j - j0];
+    const gs::ChainShape ch = gs::choose_chain(sk->rotation[j], d, kMinStride, max_steps);
+    row.a = sk->h.a[j];
+    row.b = sk->h.b[j];
+    row.a2 = sk->h.a2[j];
+    row.b2 = sk->h.b2[j];
+    row.sa = gs::mulmod61(row.a, (uint64_t)ch.stride);
+    row.sa2 = gs::mulmod61(row.a2, (uint64_t)ch.stride);
+    row.cells = cells + (size_t)j * sk->c * pitch;
+    row.stride = ch.stride;
+    row.steps = ch.steps;
+  }
+  const cudaError_t err = gs::launch_insert_chain(p, W, s);
+  if (err != cudaSuccess) return cuda_fail(err, "chained insert launch");
+  return GS_OK;
+}
+
+// How many rows (c a power of two) the accumulate pass of a group inserts directly, one reduction
+// per coordinate and row; the others go by chains, which read the error vectors once more per row.
+// Insert phase in ms, all rows direct / none:
+//   W = 1: d = 2^20 0.047 / 0.020, 25.6M 0.664 / 0.305    W = 2: 0.041 / 0.024, 0.720 / 0.458
+//   W = 4: d = 2^20 0.038 / 0.031, 2.5M 0.087 / 0.068, 25.6M 0.825 / 0.695
+//   W = 8: d = 300k 0.022 / 0.022, 2^20 0.059 / 0.049, 2.5M 0.131 / 0.126, 25.6M 1.19 / 1.26
+//   W = 16: d = 8M 0.64 / 0.85: a 64-byte cell costs one reduction as a 16-byte one does
+//   tables beyond L2: 16 workers, 7 x 2^20 cells, d = 138M 23.5 / 17.1; 8 workers, 5 x 2^21, d = 83M 5.4 / 4.6
+// Up to 2^20 updates (5 us of reductions) a second launch costs more than it saves (d = 100k, W = 4,
+// r = 5: 12 us direct, 14 us in two launches).  Gradients read from host memory are bound by the link
+// to the host, under which the direct reductions cost nothing.
+int direct_rows(const gs_sketch* sk, int64_t d, bool remote) {
+  if (d * sk->r <= kFewUpdates) return sk->r;
+  if (remote) return sk->rows_per_pass;
+  if (sk->rows_per_pass < sk->r) return 0;
+  if (sk->W == 16) return sk->r;
+  return (sk->W == 8 && d >= kDirectMinDim) ? sk->r : 0;
+}
+
 gs_status accumulate_insert_impl(gs_sketch* sk, int32_t first, int32_t n, float* const* m,
                                  float* const* e, const float* const* g, int64_t d, float rho,
-                                 cudaStream_t s) {
+                                 cudaStream_t s, bool remote = false) {
   const int W = sk->W;
   const int end = first + n;
   for (int grp = first / W; grp * W < end; ++grp) {
@@ -194,8 +262,16 @@ gs_status accumulate_insert_impl(gs_sketch* sk, int32_t first, int32_t n, float*
     p.cmask = (uint32_t)sk->c - 1;
     p.rho = rho;
     p.h = sk->h;
+    if (!sk->rotation.empty()) {
+      p.j1 = direct_rows(sk, d, remote);
+      const cudaError_t err = gs::launch_accumulate_insert(p, W, true, vec, s);
+      if (err != cudaSuccess) return cuda_fail(err, "accumulate_insert launch");
+      GS_TRY(insert_chains(sk, p.table, W, W, p.j1, p.e, nw, d, s));
+      continue;
+    }
     // first pass: accumulate and insert the first slice; later passes insert the remaining
     // slices from the updated error vectors
+    p.evict = sk->rows_per_pass < sk->r;
     bool first = true;
     for (const Pass& ps : insert_passes(sk)) {
       p.j0 = ps.j0;
@@ -228,6 +304,11 @@ gs_status insert_all_impl(gs_sketch* sk, const float* const* vec, int64_t d, cud
     p.c = (uint32_t)sk->c;
     p.cmask = (uint32_t)sk->c - 1;
     p.h = sk->h;
+    if (!sk->rotation.empty()) {
+      GS_TRY(insert_chains(sk, p.table, W, W, 0, p.e, nw, d, s));
+      continue;
+    }
+    p.evict = sk->rows_per_pass < sk->r;
     for (const Pass& ps : insert_passes(sk)) {
       p.j0 = ps.j0;
       p.j1 = ps.j1;
@@ -262,13 +343,13 @@ struct Selection {
 gs_status step_impl(gs_sketch* sk, float* const* m, float* const* e, const float* const* g,
                     int64_t d, float rho, int64_t k, int64_t* idx, float* vals, float* est,
                     void* ws, cudaStream_t s, float* weights = nullptr, float lr = 0.f,
-                    InsertMarks marks = InsertMarks(), Selection sel = Selection()) {
+                    InsertMarks marks = InsertMarks(), Selection sel = Selection(), bool remote = false) {
   const size_t bytes = (size_t)sk->groups * sk->r * sk->c * sk->W * sizeof(float) +
                        (size_t)sk->r * sk->c * sizeof(float);
   cudaError_t err = cudaMemsetAsync(sk->tables, 0, bytes, s);
   if (err != cudaSuccess) return cuda_fail(err, "zero tables");
   if ((err = mark(marks.ev[kInsertBegin], s)) != cudaSuccess) return cuda_fail(err, "event record");
-  GS_TRY(accumulate_insert_impl(sk, 0, sk->workers, m, e, g, d, rho, s));
+  GS_TRY(accumulate_insert_impl(sk, 0, sk->workers, m, e, g, d, rho, s, remote));
   if ((err = mark(marks.ev[kInsertEnd], s)) != cudaSuccess) return cuda_fail(err, "event record");
   gs::MergeParams mp;
   mp.tables = sk->tables;
@@ -418,8 +499,10 @@ gs_status check_host_step(gs_sketch* sk, float* const* momentum, float* const* e
 
 // Where the fused kernel reads each worker's host gradient: the gradient itself where the GPU
 // can address it (pinned or registered host memory, device memory, or any host memory when
-// the device has pageable-memory access), else nullptr: first copied into grad_dev[p].
-void host_sources(const gs_sketch* sk, const float* const* grad_host, std::vector<const float*>& src) {
+// the device has pageable-memory access), else nullptr: first copied into grad_dev[p].  Returns
+// whether the kernel reads some of them over the link to the host.
+bool host_sources(const gs_sketch* sk, const float* const* grad_host, std::vector<const float*>& src) {
+  bool remote = false;
   int pageable = 0;
   cudaDeviceGetAttribute(&pageable, cudaDevAttrPageableMemoryAccess, sk->device);
   src.assign((size_t)sk->workers, nullptr);
@@ -434,15 +517,19 @@ void host_sources(const gs_sketch* sk, const float* const* grad_host, std::vecto
     if (attr.type == cudaMemoryTypeHost && attr.devicePointer) direct = static_cast<const float*>(attr.devicePointer);
     else if (attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged) direct = grad_host[p];
     else if (attr.type == cudaMemoryTypeUnregistered && pageable == 1) direct = grad_host[p];
-    if (direct && aligned(direct, 4)) src[(size_t)p] = direct;
+    if (direct && aligned(direct, 4)) {
+      src[(size_t)p] = direct;
+      remote = remote || attr.type == cudaMemoryTypeHost || attr.type == cudaMemoryTypeUnregistered;
+    }
   }
+  return remote;
 }
 
 // The host step on stream s: uploads where needed, the whole step, and the download of the
 // k indices and values into the host outputs (not synchronised).
 gs_status host_step_enqueue(gs_sketch* sk, float* const* momentum, float* const* error, const float* const* grad_host,
-                            float* const* grad_dev, const std::vector<const float*>& src, int64_t d, float rho,
-                            int64_t k, int64_t* idx_host, float* vals_host, void* workspace, cudaStream_t s,
+                            float* const* grad_dev, const std::vector<const float*>& src, bool remote, int64_t d,
+                            float rho, int64_t k, int64_t* idx_host, float* vals_host, void* workspace, cudaStream_t s,
                             InsertMarks marks = InsertMarks()) {
   const size_t qbytes = gs::query_topk_workspace_bytes(d, k);
   int64_t* idx_dev = reinterpret_cast<int64_t*>(static_cast<char*>(workspace) + qbytes);
@@ -455,7 +542,7 @@ gs_status host_step_enqueue(gs_sketch* sk, float* const* momentum, float* const*
     gsrc[(size_t)p] = grad_dev[p];
   }
   GS_TRY(step_impl(sk, momentum, error, gsrc.data(), d, rho, k, idx_dev, vals_dev, nullptr, workspace, s, nullptr, 0.f,
-                   marks));
+                   marks, Selection(), remote));
   cudaError_t e = cudaMemcpyAsync(idx_host, idx_dev, (size_t)k * sizeof(int64_t), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(vals_host, vals_dev, (size_t)k * sizeof(float), cudaMemcpyDeviceToHost, s);
   if (e != cudaSuccess) return cuda_fail(e, "result download");
@@ -616,6 +703,10 @@ gs_status gs_sketch_create(int32_t r, int32_t c, uint64_t seed, int32_t workers,
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
+  std::unique_ptr<gs_sketch> sk(new gs_sketch);
+  derive_coefficients(r, seed, sk->h);
+  if (gs::is_pow2((uint32_t)c))
+    for (int j = 0; j < r; ++j) sk->rotation.push_back(gs::rotation_convergents(sk->h.a[j], (uint32_t)c));
   const int W = group_width ? group_width : choose_group_width(r, c, workers);
   const int groups = (workers + W - 1) / W;
   const size_t table_floats = (size_t)groups * r * c * W;
@@ -632,7 +723,6 @@ gs_status gs_sketch_create(int32_t r, int32_t c, uint64_t seed, int32_t workers,
     cudaFree(mem);
     return cuda_fail(e, "cudaMemset");
   }
-  gs_sketch* sk = new gs_sketch;
   sk->r = r;
   sk->c = c;
   sk->workers = workers;
@@ -640,11 +730,10 @@ gs_status gs_sketch_create(int32_t r, int32_t c, uint64_t seed, int32_t workers,
   sk->groups = groups;
   sk->rows_per_pass = choose_rows_per_pass(r, c, W);
   sk->seed = seed;
-  derive_coefficients(r, seed, sk->h);
   sk->tables = mem;
   sk->merged = mem + table_floats;
   sk->device = dev;
-  *out = sk;
+  *out = sk.release();
   return ok();
   GS_GUARD_END
 }
@@ -718,11 +807,14 @@ gs_status gs_sketch_insert(gs_sketch* sk, int32_t worker, const float* vec, int6
   GS_TRY(check_vec(vec, "vec"));
   GS_TRY(check_d(d));
   if (worker < 0 || worker >= sk->workers) return fail(GS_ERR_INVALID_ARG, "worker out of range");
+  const int W = sk->W;
+  float* const table = sk->tables + (size_t)(worker / W) * sk->r * sk->c * W;
+  if (!sk->rotation.empty())
+    return insert_chains(sk, table + worker % W, W, 1, 0, &vec, 1, d, as_stream(stream));
   gs::InsertParams p;
   std::memset(&p, 0, sizeof(p));
-  const int W = sk->W;
   p.e[0] = const_cast<float*>(vec);
-  p.table = sk->tables + (size_t)(worker / W) * sk->r * sk->c * W;
+  p.table = table;
   p.lane = worker % W;
   p.d = d;
   p.nw = 1;
@@ -1102,9 +1194,10 @@ gs_status gs_step_host(gs_sketch* sk, float* const* momentum, float* const* erro
   GS_TRY(check_host_step(sk, momentum, error, grad_host, grad_dev, d, k, idx_host, vals_host, workspace,
                          workspace_bytes));
   std::vector<const float*> src;
-  host_sources(sk, grad_host, src);
+  const bool remote = host_sources(sk, grad_host, src);
   cudaStream_t s = as_stream(stream);
-  GS_TRY(host_step_enqueue(sk, momentum, error, grad_host, grad_dev, src, d, rho, k, idx_host, vals_host, workspace, s));
+  GS_TRY(host_step_enqueue(sk, momentum, error, grad_host, grad_dev, src, remote, d, rho, k, idx_host, vals_host, workspace,
+                           s));
   cudaError_t e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "result download");
   return GS_OK;
@@ -1158,9 +1251,9 @@ gs_status gs_step_host_plan_create(gs_sketch* sk, float* const* momentum, float*
   GS_TRY(check_host_step(sk, momentum, error, grad_host, grad_dev, d, k, idx_host, vals_host, workspace,
                          workspace_bytes));
   std::vector<const float*> src;
-  host_sources(sk, grad_host, src);
+  const bool remote = host_sources(sk, grad_host, src);
   return capture_plan(sk->device, flags, plan_out, [&](cudaStream_t s, InsertMarks marks) {
-    return host_step_enqueue(sk, momentum, error, grad_host, grad_dev, src, d, rho, k, idx_host, vals_host, workspace,
+    return host_step_enqueue(sk, momentum, error, grad_host, grad_dev, src, remote, d, rho, k, idx_host, vals_host, workspace,
                              s, marks);
   });
   GS_GUARD_END
@@ -1299,6 +1392,7 @@ gs_status gs_insert_request_ceiling(gs_sketch* sk, int64_t d, void* window, size
     p.c = (uint32_t)sk->c;
     p.cmask = (uint32_t)sk->c - 1;
     p.rho = 0.9f;
+    p.evict = sk->rows_per_pass < sk->r;
     p.winmask = GS_CEILING_WINDOW_FLOATS - 1;
     p.h = sk->h;
     bool first = true;

@@ -70,11 +70,12 @@ __device__ __forceinline__ void red_add_v4(float* p, float v0, float v1, float v
 }
 
 // ---- L2 eviction priorities -------------------------------------------------------------
-// Cache policies for the fused insert: its vector streams are read or written once
-// (evict_first, not allocated in L1), while the sketch table receives every reduction and
-// should stay in L2 (evict_last).  Measured on the BERT-large-sized table (64 MiB row slices
-// next to 8 workers' streams): one group's five row passes 21.9 ms with these policies against
-// 25.0 ms without; neutral at the other sizes.
+// Cache policies for the insert: the sketch table receives every reduction and should stay in L2
+// (evict_last).  Vector streams are marked evict_first only where the table does not fit L2 beside
+// them (64 MiB row slices and 8 workers' streams: five row passes 21.9 ms with both policies, 25.0
+// without).  Elsewhere evict_first costs: a line that two warps share, as every line of a vector
+// that does not start on a 128-byte boundary does, may be evicted half written.  Accumulating 8
+// vectors of 25,557,032, 32 bytes off such a boundary: 0.645 ms without the mark, 0.745 with it.
 __device__ __forceinline__ uint64_t policy_evict_first() {
   uint64_t pol;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
@@ -84,6 +85,16 @@ __device__ __forceinline__ uint64_t policy_evict_last() {
   uint64_t pol;
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
   return pol;
+}
+__device__ __forceinline__ uint64_t policy_normal() {
+  uint64_t pol;
+  asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
+  return pol;
+}
+__device__ __forceinline__ float ld_hinted(const float* p, uint64_t pol) {
+  float v;
+  asm volatile("ld.global.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
+  return v;
 }
 __device__ __forceinline__ float4 ld_stream(const float* p, uint64_t pol) {
   float4 v;
@@ -116,8 +127,31 @@ struct InsertParams {
   int32_t j0, j1;    // rows inserted by this launch: [j0, j1)
   uint32_t c, cmask;
   float rho;
+  int32_t evict;     // the table does not fit L2 beside the streams: mark these evict_first
   int64_t winmask;   // request-ceiling probe only: vector offsets are taken modulo winmask + 1
   HashCoeffs h;
+};
+
+// Rows inserted by chains of coordinates (k_insert_chain), in launch order.
+struct ChainRow {
+  uint64_t a, b, a2, b2;  // the row's hash coefficients
+  uint64_t sa, sa2;       // a * stride and a2 * stride mod p: one step along a chain
+  float* cells;           // the row's cells, ChainParams::pitch floats apart
+  int64_t stride;         // coordinates between two steps of a chain
+  int32_t steps;          // coordinates of a chain
+  uint32_t tiles;         // CTAs across the stride
+  uint32_t first_block;   // first CTA of this row
+};
+
+struct ChainParams {
+  const float* e[kMaxGroup];
+  int64_t d;
+  uint32_t cmask;
+  int32_t nw;             // vectors inserted
+  int32_t pitch;          // floats between two cells of a row
+  int32_t nrows;
+  int32_t resident;       // the vectors fit L2 between two rows
+  ChainRow row[GS_MAX_ROWS];
 };
 
 struct MergeParams {
@@ -160,6 +194,10 @@ cudaError_t launch_accumulate(float* u, float* e, const float* g, int64_t d, flo
 // acc: accumulate (read g, u, e; write u, e) before inserting; otherwise insert e as it is.
 cudaError_t launch_accumulate_insert(const InsertParams& p, int W, bool acc, bool vec, cudaStream_t s);
 cudaError_t launch_insert_lane(const InsertParams& p, int W, cudaStream_t s);
+// Inserts the vectors p.e[0..nw) into the p.nrows rows of p.row (c a power of two; the strides and
+// steps chosen by the caller, tiles and first_block filled in here).  W in {1, 2, 4, 8, 16}: workers
+// per cell written; p.pitch == W unless W == 1.
+cudaError_t launch_insert_chain(ChainParams& p, int W, cudaStream_t s);
 // The fused insert's instruction stream with every vector access at offset i & p.winmask (the
 // vectors are windows of winmask + 1 floats, 16-byte aligned): the same loads, stores and
 // cell reductions, with the streams held in L2.  W in {4, 8, 16}, c a power of two.
