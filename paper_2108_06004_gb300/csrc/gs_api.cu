@@ -20,8 +20,9 @@ struct gs_sketch {
   float* tables;  // groups * r*c*W
   float* merged;  // r*c
   int device;
-  // c a power of two: the convergents of every row's rotation (chain_plan.h), else empty
-  std::vector<std::vector<gs::Convergent>> rotation;
+  // c a power of two: the convergents of every row's rotation (chain_plan.h) by one coordinate and
+  // by a quad of four, else empty
+  std::vector<std::vector<gs::Convergent>> rotation, quad_rotation;
 };
 
 // Events recorded between the phases of a step while it is captured into a plan, where each
@@ -101,8 +102,8 @@ constexpr size_t kPassBudget = size_t(48) << 20;
 constexpr size_t kResidentBytes = size_t(64) << 20;
 // Shortest stride of a chain: 16 CTAs of chains, so that the last CTA's idle lanes stay few.
 constexpr int64_t kMinStride = 4096;
-// 8-wide groups insert directly from this length on.
-constexpr int64_t kDirectMinDim = int64_t(1) << 22;
+// The accumulate pass walks chains from this length on.
+constexpr int64_t kWalkMinDim = int64_t(1) << 22;
 // Up to this many cell updates per worker every row is inserted directly.
 constexpr int64_t kFewUpdates = int64_t(1) << 20;
 
@@ -217,23 +218,35 @@ gs_status insert_chains(const gs_sketch* sk, float* cells, int pitch, int W, int
   return GS_OK;
 }
 
-// How many rows (c a power of two) the accumulate pass of a group inserts directly, one reduction
-// per coordinate and row; the others go by chains, which read the error vectors once more per row.
-// Insert phase in ms, all rows direct / none:
-//   W = 1: d = 2^20 0.047 / 0.020, 25.6M 0.664 / 0.305    W = 2: 0.041 / 0.024, 0.720 / 0.458
-//   W = 4: d = 2^20 0.038 / 0.031, 2.5M 0.087 / 0.068, 25.6M 0.825 / 0.695
-//   W = 8: d = 300k 0.022 / 0.022, 2^20 0.059 / 0.049, 2.5M 0.131 / 0.126, 25.6M 1.19 / 1.26
-//   W = 16: d = 8M 0.64 / 0.85: a 64-byte cell costs one reduction as a 16-byte one does
-//   tables beyond L2: 16 workers, 7 x 2^20 cells, d = 138M 23.5 / 17.1; 8 workers, 5 x 2^21, d = 83M 5.4 / 4.6
+// What the accumulate pass of a group inserts (c a power of two): rows [0, rows), along chains
+// that serve row 0 (walk) or one reduction per coordinate and row; the other rows go by
+// insert_chains, which reads the error vectors once more per row.
+struct MainPass {
+  int rows;
+  bool walk;
+};
+
+// Insert phase in ms, r = 5: all rows directly / none, all by insert_chains / walking with W/2 rows
+//   W = 1: d = 2^20 0.047 / 0.020, 4.2M 0.114 / 0.051 / 0.051, 25.6M 0.664 / 0.306 / 0.274
+//   W = 2: d = 2^20 0.041 / 0.024, 25.6M 0.720 / 0.458 / 0.411
+//   W = 4: d = 2^20 0.038 / 0.031, 4.2M 0.133 / 0.099 / 0.102, 25.6M 0.825 / 0.695 / 0.638
+//   W = 8: d = 300k 0.022 / 0.022, 2^20 0.059 / 0.049, 2.5M 0.131 / 0.126 / 0.128,
+//          11.2M 0.616 / 0.574 / 0.495, 25.6M 1.33 / 1.26 / 1.09
+//   W = 16: d = 8M 0.73 / 0.85 / 0.62 with all rows (a 64-byte cell costs one reduction, as a
+//          16-byte one does, while reading the vectors again costs four times as much)
+//   16 workers, 7 x 2^20 cells (32 MiB a row and group), d = 138M: 23.5 / 17.1 / 16.6 with one row
+//   16 workers, 5 x 2^21 (64 MiB a row), d = 83M: 10.6 / 9.1 / 9.3 with one row
 // Up to 2^20 updates (5 us of reductions) a second launch costs more than it saves (d = 100k, W = 4,
 // r = 5: 12 us direct, 14 us in two launches).  Gradients read from host memory are bound by the link
 // to the host, under which the direct reductions cost nothing.
-int direct_rows(const gs_sketch* sk, int64_t d, bool remote) {
-  if (d * sk->r <= kFewUpdates) return sk->r;
-  if (remote) return sk->rows_per_pass;
-  if (sk->rows_per_pass < sk->r) return 0;
-  if (sk->W == 16) return sk->r;
-  return (sk->W == 8 && d >= kDirectMinDim) ? sk->r : 0;
+MainPass main_pass(const gs_sketch* sk, int64_t d, bool remote) {
+  if (d * sk->r <= kFewUpdates) return {sk->r, false};
+  if (remote) return {sk->rows_per_pass, false};
+  const size_t row_bytes = (size_t)sk->c * sk->W * sizeof(float);
+  if (d < kWalkMinDim) return {sk->W == 16 ? sk->rows_per_pass : 0, false};
+  const int rows = sk->W == 16 ? sk->r : std::max(1, sk->W / 2);
+  const int rows_in_l2 = (int)std::min<size_t>(kPassBudget / row_bytes, (size_t)sk->r);
+  return {std::min(rows, rows_in_l2), rows_in_l2 > 0};
 }
 
 gs_status accumulate_insert_impl(gs_sketch* sk, int32_t first, int32_t n, float* const* m,
@@ -263,8 +276,18 @@ gs_status accumulate_insert_impl(gs_sketch* sk, int32_t first, int32_t n, float*
     p.rho = rho;
     p.h = sk->h;
     if (!sk->rotation.empty()) {
-      p.j1 = direct_rows(sk, d, remote);
-      const cudaError_t err = gs::launch_accumulate_insert(p, W, true, vec, s);
+      const MainPass mp = main_pass(sk, d, remote);
+      p.j1 = mp.rows;
+      cudaError_t err;
+      if (mp.walk) {
+        // chains of at most 12 quads and one and a half waves of 768 threads per SM
+        const int64_t nq = (d + 3) / 4, lanes = (int64_t)gs::device_info().sms * 768 * 3 / 2;
+        const int64_t max_steps = std::min<int64_t>(12, std::max<int64_t>(1, nq * std::max(1, W / 4) / lanes));
+        const gs::ChainShape ch = gs::choose_chain(sk->quad_rotation[0], nq, kMinStride / 4, max_steps);
+        err = gs::launch_accumulate_chain(p, gs::QuadWalk{ch.stride, ch.steps, 0}, W, vec, s);
+      } else {
+        err = gs::launch_accumulate_insert(p, W, true, vec, s);
+      }
       if (err != cudaSuccess) return cuda_fail(err, "accumulate_insert launch");
       GS_TRY(insert_chains(sk, p.table, W, W, p.j1, p.e, nw, d, s));
       continue;
@@ -706,7 +729,10 @@ gs_status gs_sketch_create(int32_t r, int32_t c, uint64_t seed, int32_t workers,
   std::unique_ptr<gs_sketch> sk(new gs_sketch);
   derive_coefficients(r, seed, sk->h);
   if (gs::is_pow2((uint32_t)c))
-    for (int j = 0; j < r; ++j) sk->rotation.push_back(gs::rotation_convergents(sk->h.a[j], (uint32_t)c));
+    for (int j = 0; j < r; ++j) {
+      sk->rotation.push_back(gs::rotation_convergents(sk->h.a[j], (uint32_t)c));
+      sk->quad_rotation.push_back(gs::rotation_convergents(gs::mulmod61(4, sk->h.a[j]), (uint32_t)c));
+    }
   const int W = group_width ? group_width : choose_group_width(r, c, workers);
   const int groups = (workers + W - 1) / W;
   const size_t table_floats = (size_t)groups * r * c * W;

@@ -96,6 +96,13 @@ __device__ __forceinline__ float ld_hinted(const float* p, uint64_t pol) {
   asm volatile("ld.global.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
   return v;
 }
+__device__ __forceinline__ float4 ld_hinted4(const float* p, uint64_t pol) {
+  float4 v;
+  asm volatile("ld.global.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(p), "l"(pol));
+  return v;
+}
 __device__ __forceinline__ float4 ld_stream(const float* p, uint64_t pol) {
   float4 v;
   asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
@@ -141,6 +148,13 @@ struct ChainRow {
   int32_t steps;          // coordinates of a chain
   uint32_t tiles;         // CTAs across the stride
   uint32_t first_block;   // first CTA of this row
+};
+
+// How k_accumulate_chain walks the coordinates: chains of `steps` quads, `stride` quads apart.
+struct QuadWalk {
+  int64_t stride;
+  int32_t steps;
+  uint32_t tiles;  // CTAs across the stride
 };
 
 struct ChainParams {
@@ -193,6 +207,9 @@ cudaError_t launch_accumulate(float* u, float* e, const float* g, int64_t d, flo
                               cudaStream_t s);
 // acc: accumulate (read g, u, e; write u, e) before inserting; otherwise insert e as it is.
 cudaError_t launch_accumulate_insert(const InsertParams& p, int W, bool acc, bool vec, cudaStream_t s);
+// The accumulate pass with rows [p.j0, p.j1) inserted (at least one; c a power of two), walking the
+// chains of `wk` (tiles filled in here), along which row p.j0 keeps its buckets.
+cudaError_t launch_accumulate_chain(const InsertParams& p, QuadWalk wk, int W, bool vec, cudaStream_t s);
 cudaError_t launch_insert_lane(const InsertParams& p, int W, cudaStream_t s);
 // Inserts the vectors p.e[0..nw) into the p.nrows rows of p.row (c a power of two; the strides and
 // steps chosen by the caller, tiles and first_block filled in here).  W in {1, 2, 4, 8, 16}: workers

@@ -228,6 +228,123 @@ __global__ void __launch_bounds__(kBlock) k_accumulate_insert_coop(const __grid_
   }
 }
 
+// The accumulate pass along chains of quads (c a power of two): row prm.j0 keeps its buckets along a
+// chain, so its values are summed in registers and its cells updated only when a bucket changes;
+// rows prm.j0 + 1 .. prm.j1 - 1 take one reduction per coordinate as above.  Every lane holds one
+// quad of min(W, 4) workers.  At W = 8 the pass is bound by HBM with up to three such rows
+// (0.72, 0.75, 0.83 ms for 1, 2, 3 rows of 8 workers at d = 25,557,032; 0.94 and 1.08 ms for 4 and
+// 5, where the reductions take over).  Loads go through L1, where neighbouring warps find the rest
+// of the lines they share when a vector does not start on a 128-byte boundary: the times are the
+// same for both, while k_accumulate_insert_coop takes 0.83 ms for three rows of aligned vectors and
+// 0.95 ms off the boundary.  Staging the next step in shared memory by cp.async was slower (0.88 ms
+// for one row): it halves the resident warps.
+template <int N>
+__device__ __forceinline__ void red_lane(float* cell, const float (&v)[N], uint64_t pol) {
+  if constexpr (N == 4) red_add_v4_keep(cell, v[0], v[1], v[2], v[3], pol);
+  else if constexpr (N == 2) red_add_v2(cell, v[0], v[1]);
+  else red_add_f32(cell, v[0]);
+}
+
+template <int W, bool VEC>
+__global__ void __launch_bounds__(kBlock, 3) k_accumulate_chain(const __grid_constant__ InsertParams prm,
+                                                                const __grid_constant__ QuadWalk wk) {
+  grid_begin();
+  constexpr int G = W >= 4 ? W / 4 : 1;  // lanes that share a quad
+  constexpr int N = W >= 4 ? 4 : W;      // workers per lane
+  constexpr uint32_t kNoCell = 0xFFFFFFFFu;
+  const int sub = threadIdx.x % G;
+  const int64_t d = prm.d;
+  const int64_t nq = (d + 3) / 4;
+  const uint32_t seg = blockIdx.x / wk.tiles;
+  const int64_t tq = (int64_t)(blockIdx.x - seg * wk.tiles) * (kBlock / G) + threadIdx.x / G;
+  int64_t q = (int64_t)seg * wk.steps * wk.stride + tq;
+  if (tq >= wk.stride || q >= nq) return;
+  const uint64_t pol = policy_normal(), pol_table = policy_evict_last();
+  float acc[4][N];
+  uint32_t cur[4];
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    cur[t] = kNoCell;
+#pragma unroll
+    for (int w = 0; w < N; ++w) acc[t][w] = 0.f;
+  }
+  float* const crow = prm.table + (size_t)prm.j0 * prm.c * W + sub * 4;
+#pragma unroll 1
+  for (int n = wk.steps; n > 0 && q < nq; --n, q += wk.stride) {
+    const int64_t i0 = q * 4;
+    const int tmax = (d - i0 < 4) ? (int)(d - i0) : 4;
+    float ev[N][4];
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const int w = sub * 4 + k;
+      if (w >= prm.nw) {
+#pragma unroll
+        for (int t = 0; t < 4; ++t) ev[k][t] = 0.f;
+      } else if (VEC && tmax == 4) {
+        float4 e4 = ld_hinted4(prm.e[w] + i0, pol);
+        const float4 g4 = ld_hinted4(prm.g[w] + i0, pol);
+        float4 u4 = ld_hinted4(prm.u[w] + i0, pol);
+        acc1(prm.rho, u4.x, e4.x, g4.x);
+        acc1(prm.rho, u4.y, e4.y, g4.y);
+        acc1(prm.rho, u4.z, e4.z, g4.z);
+        acc1(prm.rho, u4.w, e4.w, g4.w);
+        st_stream(prm.u[w] + i0, u4, pol);
+        st_stream(prm.e[w] + i0, e4, pol);
+        ev[k][0] = e4.x;
+        ev[k][1] = e4.y;
+        ev[k][2] = e4.z;
+        ev[k][3] = e4.w;
+      } else {
+        load_lane<true, false>(prm, w, i0, d, ev[k]);
+      }
+    }
+    {
+      const uint64_t a = prm.h.a[prm.j0], a2 = prm.h.a2[prm.j0];
+      uint64_t x = affine61(a, prm.h.b[prm.j0], (uint32_t)i0);
+      uint64_t y = affine61(a2, prm.h.b2[prm.j0], (uint32_t)i0);
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        if (t < tmax) {
+          const uint32_t b = (uint32_t)x & prm.cmask;
+          const float sg = __uint_as_float(0x3F800000u | signbit_of(y));
+          if (b != cur[t]) {
+            if (cur[t] != kNoCell) red_lane<N>(crow + (size_t)cur[t] * W, acc[t], pol_table);
+            cur[t] = b;
+#pragma unroll
+            for (int w = 0; w < N; ++w) acc[t][w] = 0.f;
+          }
+#pragma unroll
+          for (int w = 0; w < N; ++w) acc[t][w] = fmaf(ev[w][t], sg, acc[t][w]);  // sg is +-1
+          x = step61(x, a);
+          y = step61(y, a2);
+        }
+      }
+    }
+#pragma unroll 1
+    for (int j = prm.j0 + 1; j < prm.j1; ++j) {
+      const uint64_t a = prm.h.a[j], a2 = prm.h.a2[j];
+      uint64_t x = affine61(a, prm.h.b[j], (uint32_t)i0);
+      uint64_t y = affine61(a2, prm.h.b2[j], (uint32_t)i0);
+      float* row = prm.table + (size_t)j * prm.c * W + sub * 4;
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        if (t < tmax) {
+          const uint32_t sb = signbit_of(y);
+          float v[N];
+#pragma unroll
+          for (int w = 0; w < N; ++w) v[w] = apply_sign(ev[w][t], sb);
+          red_lane<N>(row + (size_t)((uint32_t)x & prm.cmask) * W, v, pol_table);
+          x = step61(x, a);
+          y = step61(y, a2);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < 4; ++t)
+    if (cur[t] != kNoCell) red_lane<N>(crow + (size_t)cur[t] * W, acc[t], pol_table);
+}
+
 // Insert one vector (prm.e[0]) into lane prm.lane of a W-wide group table, c not a power of two.
 __global__ void __launch_bounds__(kBlock) k_insert_lane(const __grid_constant__ InsertParams prm, int W) {
   grid_begin();
@@ -543,6 +660,28 @@ cudaError_t launch_insert_staged(const InsertParams& p, int W, cudaStream_t s) {
     case 4: return pow2 ? launch_staged_t<4, true>(p, W, s) : launch_staged_t<4, false>(p, W, s);
     case 2: return pow2 ? launch_staged_t<2, true>(p, W, s) : launch_staged_t<2, false>(p, W, s);
     case 1: return pow2 ? launch_staged_t<1, true>(p, W, s) : launch_staged_t<1, false>(p, W, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+template <int W>
+cudaError_t launch_acc_chain_w(const InsertParams& p, QuadWalk wk, bool vec, cudaStream_t s) {
+  constexpr int G = W >= 4 ? W / 4 : 1;
+  const int64_t nq = (p.d + 3) / 4, span = wk.stride * wk.steps;
+  wk.tiles = (uint32_t)((wk.stride + kBlock / G - 1) / (kBlock / G));
+  const uint32_t blocks = wk.tiles * (uint32_t)((nq + span - 1) / span);
+  if (vec) launch(k_accumulate_chain<W, true>, blocks, kBlock, s, p, wk);
+  else launch(k_accumulate_chain<W, false>, blocks, kBlock, s, p, wk);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_accumulate_chain(const InsertParams& p, QuadWalk wk, int W, bool vec, cudaStream_t s) {
+  switch (W) {
+    case 1: return launch_acc_chain_w<1>(p, wk, vec, s);
+    case 2: return launch_acc_chain_w<2>(p, wk, vec, s);
+    case 4: return launch_acc_chain_w<4>(p, wk, vec, s);
+    case 8: return launch_acc_chain_w<8>(p, wk, vec, s);
+    case 16: return launch_acc_chain_w<16>(p, wk, vec, s);
     default: return cudaErrorInvalidValue;
   }
 }
