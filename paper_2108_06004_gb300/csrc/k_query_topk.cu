@@ -30,10 +30,12 @@
 // With the fixed scratch (gs_query_topk_noalloc), which cannot hold candidate lists, the
 // levels 2 and 3 and the final selection read est in full passes (k_hist, k_count, k_write).
 #include <cmath>
+#include <cstring>
 #include <mutex>
 
 #include <cuda.h>
 
+#include "chain_plan.h"
 #include "gs_common.cuh"
 
 namespace gs {
@@ -66,7 +68,7 @@ inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 __device__ __forceinline__ uint32_t key_of(float v) { return __float_as_uint(v) & 0x7FFFFFFFu; }
 
-// The query's hash arithmetic, without compares (the query is bound by its integer work).
+// The hash arithmetic of k_query and k_qsample, without compares.
 // For s < 2^62 - 1, s mod p is s - p when s >= p and s otherwise; s >= p exactly when bit 61
 // of s + 1 is set, and then s - p = (s + 1) - 2^61 = (s + 1) & p.  So for s < 2p:
 //   s mod p = (s + ((s + 1) >> 61)) & p.
@@ -83,6 +85,54 @@ __device__ __forceinline__ uint64_t affine61_nb(uint64_t a, uint64_t b, uint32_t
   const uint64_t s = (p1 >> 29) + ((p1 & ((1ull << 29) - 1)) << 32) + fold61(p0) + b;
   return reduce61(fold61(s));
 }
+
+// The hash arithmetic of k_query_bits, which is bound by its integer instructions.  (k_query is bound
+// by its reads; with this form it took 4 % longer.)  A hash value x in [0, p),
+// p = 2^61 - 1, is held as Y = 8 (x + 1), which lies in [8, 2^64 - 8].  For a residue s the 64-bit sum
+// Y + 8 s = 8 (x + s + 1) overflows exactly when x + s >= p, and then (x + s) mod p is represented by
+// the wrapped sum plus 8, since 8 p = 2^64 - 8.  So an addition and its carry-out reduce exactly,
+// without a compare, and the low word of Y alone gives the bucket and the sign.
+struct Rot {
+  uint32_t lo, hi;
+};
+
+// The representation of (x + s) mod p from that of x; s8 = 8 s, s in [0, p).
+__device__ __forceinline__ Rot rot_add(Rot y, uint64_t s8) {
+  uint32_t lo, hi, carry;
+  asm("add.cc.u32 %0, %3, %5;\n\taddc.cc.u32 %1, %4, %6;\n\taddc.u32 %2, 0, 0;"
+      : "=r"(lo), "=r"(hi), "=r"(carry)
+      : "r"(y.lo), "r"(y.hi), "r"((uint32_t)s8), "r"((uint32_t)(s8 >> 32)));
+  Rot out;
+  asm("add.cc.u32 %0, %2, %4;\n\taddc.u32 %1, %3, 0;" : "=r"(out.lo), "=r"(out.hi) : "r"(lo), "r"(hi), "r"(8u * carry));
+  return out;
+}
+
+// The low word of rot_add.
+__device__ __forceinline__ uint32_t rot_add_lo(Rot y, uint64_t s8) {
+  uint32_t lo, carry;
+  asm("{\n\t.reg .u32 hi;\n\tadd.cc.u32 %0, %2, %4;\n\taddc.cc.u32 hi, %3, %5;\n\taddc.u32 %1, 0, 0;\n\t}"
+      : "=r"(lo), "=r"(carry)
+      : "r"(y.lo), "r"(y.hi), "r"((uint32_t)s8), "r"((uint32_t)(s8 >> 32)));
+  return lo + 8u * carry;
+}
+
+// The representation of a i mod p, from a8 = 8 a, for i < 2^32: 8 a i = h 2^64 + l with h < 2^32, and
+// 2^64 is 8 modulo 2^64 - 8, so l + 8 h + 8 with its carry folded in as above (l / 8 + h < 2 p).
+__device__ __forceinline__ Rot rot_mul(uint64_t a8, uint32_t i) {
+  const uint64_t w = (uint64_t)(uint32_t)a8 * i;
+  const uint64_t z = (uint64_t)(uint32_t)(a8 >> 32) * i + (w >> 32);
+  return rot_add(Rot{(uint32_t)w, (uint32_t)z}, 8ull * (uint32_t)(z >> 32) + 8ull);
+}
+
+// The representation of (a i + b) mod p, and its low word.
+__device__ __forceinline__ Rot rot_at(uint64_t a8, uint64_t b8, uint32_t i) { return rot_add(rot_mul(a8, i), b8); }
+__device__ __forceinline__ uint32_t rot_at_lo(uint64_t a8, uint64_t b8, uint32_t i) {
+  return rot_add_lo(rot_mul(a8, i), b8);
+}
+
+// From the low word: the bucket for c a power of two, and the sign bit (bit 31 set when x is odd).
+__device__ __forceinline__ uint32_t rot_bucket(uint32_t lo, uint32_t cmask) { return ((lo >> 3) - 1u) & cmask; }
+__device__ __forceinline__ uint32_t rot_signbit(uint32_t lo) { return (~lo & 8u) << 28; }
 
 // Warp-aggregated shared-memory histogram update; every lane of the warp must call it.
 __device__ __forceinline__ void hist_add(uint32_t* sh, uint32_t bin) {
@@ -240,7 +290,20 @@ struct QueryParams {
   const double* theta;  // HEAVYMIX: the threshold l2sq / k of H
   uint64_t fill_seed;   // HEAVYMIX: the seed of the random fill
   HashCoeffs h;
+  HashCoeffs h8;        // 8 a, 8 b, 8 a', 8 b' of every row
+  uint64_t qa[GS_MAX_ROWS / 2 + 1][3];  // 8 (t a mod p), t = 1, 2, 3, of the first rows
 };
+
+// The low word for coordinate t of a quad, from its first coordinate.
+__device__ __forceinline__ uint32_t quad_lo(Rot y, const uint64_t (&step)[3], int t) {
+  return t == 0 ? y.lo : rot_add_lo(y, step[t - 1]);
+}
+
+// The signed cell of row j for coordinate i.
+__device__ __forceinline__ float signed_cell(const QueryParams& prm, int j, uint32_t i) {
+  const uint32_t x = rot_at_lo(prm.h8.a[j], prm.h8.b[j], i), y = rot_at_lo(prm.h8.a2[j], prm.h8.b2[j], i);
+  return apply_sign(__ldg(prm.T + (size_t)j * prm.c + rot_bucket(x, prm.cmask)), rot_signbit(y));
+}
 
 // Row pruning.  With f = r/2 + 1: if at least f of a coordinate's r signed cells are < t and
 // at least f are > -t, then -t < est < t.  For odd r the median is the f-th smallest and the
@@ -396,56 +459,118 @@ __global__ void __launch_bounds__(kBlock, R <= 7 ? 4 : 1) k_query(const __grid_c
 
 // ---- the pruning query with the first rows classified in shared memory ---------------------
 // The settle rule needs, for each of the first f = r/2 + 1 cells of a coordinate, only which side
-// of the prune key t its value lies on.  For a row that is a class per table cell, two bits:
-// whether T counts below t and whether it counts above -t (3 for |T| < t, 1 for T >= t, 2 for
-// T <= -t, 0 for NaN); the sign hash of the coordinate swaps the two bits.
-// Where the classes of the first f rows fit in shared memory (2 bits per cell), k_pbits writes
-// them once per query and k_query_bits looks them up instead of reading those cells from L2.  A
-// coordinate that settles within the first f rows then reads no cell at all; one that examines
-// later rows reads those cells as k_query does; one that does not settle reads every cell for
-// its full median.  The rows examined, the stops and the estimates are the same as k_query's.
-constexpr uint32_t kBitsBytes = 192u << 10;   // dynamic shared memory for the classes
+// of the prune key t its value lies on: whether it counts below t, above -t, or both (|T| < t: the
+// cell is inside).  That takes two bits per table cell: one says whether the cell is inside, the
+// other, for the others, on which side it lies; the coordinate's sign hash swaps the sides.
+// Where the bits of the first f rows fit in shared memory, k_pbits writes them once per query and
+// k_query_bits looks them up instead of reading those cells from L2.  A coordinate that settles
+// within the first f rows then reads no cell at all; one that examines later rows reads those
+// cells as k_query does; one that does not settle reads every cell for its full median.  The rows
+// examined, the stops and the estimates are the same as k_query's.
+//
+// The kernel sorts its coordinates by the work that they need, so that warps stay full.
+//   1. f rows settle a coordinate exactly when all f cells are inside, whatever the signs: four
+//      coordinates per lane, only the buckets of the first f rows, whose hash comes from a form
+//      that needs few instructions (rot_add).  The others are queued, per warp.
+//   2. With one cell of the first f outside, the next row settles a coordinate exactly when its
+//      cell is inside, again whatever the signs: 32 such coordinates at a time, one per lane, one
+//      bucket and one cell read each.
+//   3. What is left is resolved from its signs and all further rows, 32 coordinates at a time.
+// Integer instructions bound it.  d = 25,557,032, r = 5, c = 2^18: 0.098 ms, and 0.110 in HEAVYMIX
+// mode (which evaluates the fill order of every coordinate); one kernel for all coordinates, four per
+// lane, took 0.267, and 0.344 with k_query in HEAVYMIX mode.  Part 3 without part 2 takes 0.145.
+constexpr uint32_t kBitsBytes = 192u << 10;   // dynamic shared memory for the bits
 
 constexpr int kBitsBlock = 1024;              // one CTA of 32 warps per SM
+// Queue entries per warp.  Queue 2 grows from the front, queue 3 from the back; each keeps at most
+// 31 entries from one grid stride to the next, which adds at most 128.
+constexpr int kQueue = 192;
 
-// The class as two bits: bit 1 set when the cell counts below t (T < t), bit 0 when it counts
-// above -t (T > -t): 3 for |T| < t, 1 for T >= t, 2 for T <= -t, 0 for NaN.
-__device__ __forceinline__ uint32_t cell_class(float v, uint32_t pk) {
-  const uint32_t b = __float_as_uint(v), key = b & 0x7FFFFFFFu;
-  if (key > 0x7F800000u) return 0u;
-  if (key < pk) return 3u;
-  return (b >> 31) ? 2u : 1u;
-}
+// 8 (n a mod p) of the first r/2 + 1 rows for the n coordinates of one grid stride.
+struct GridSteps {
+  uint64_t a[GS_MAX_ROWS / 2 + 1];
+};
 
-// Word w holds the classes of cells 16 w .. 16 w + 15 of the first rows of the row-major merged
-// table, cell 16 w + u at bits 2u, 2u + 1.  nwords = f * c / 16.
-__global__ void __launch_bounds__(kBlock) k_pbits(const float* __restrict__ T, int64_t nwords,
+// The bits of the first kf rows: kf * c / 32 words that tell inside from outside, then as many that
+// tell the side of an outside cell (set: T <= -t).  Bit n mod 32 of word n / 32 of a row belongs to
+// the cell of bucket n - 1 mod c: its place (x + 1) mod c is what the hash gives first.
+__global__ void __launch_bounds__(kBlock) k_pbits(const float* __restrict__ T, uint32_t c, int64_t nwords,
                                                   const SelectState* st, uint32_t* __restrict__ words) {
   grid_begin();
   const uint32_t pk = __ldcg(&st->prune_key);
-  for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < nwords; w += (int64_t)gridDim.x * blockDim.x) {
-    const float4* src = reinterpret_cast<const float4*>(T) + 4 * w;
-    uint32_t out = 0;
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x / 32);
+  constexpr int kN = 4;  // words of a warp in flight
+  for (int64_t w0 = (int64_t)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); w0 < nwords; w0 += kN * warps) {
+    float v[kN];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float4 v = __ldg(src + q);
-      out |= (cell_class(v.x, pk) | cell_class(v.y, pk) << 2 | cell_class(v.z, pk) << 4 | cell_class(v.w, pk) << 6)
-             << (8 * q);
+    for (int u = 0; u < kN; ++u) {
+      const uint32_t w = (uint32_t)(w0 + u * warps);
+      const uint32_t j = w / (c / 32), n = (w - j * (c / 32)) * 32 + lane;
+      v[u] = w0 + u * warps < nwords ? __ldg(T + (size_t)j * c + ((n - 1u) & (c - 1u))) : 0.f;
     }
-    words[w] = out;
+#pragma unroll
+    for (int u = 0; u < kN; ++u) {
+      const uint32_t in = __ballot_sync(kFull, key_of(v[u]) < pk);
+      const uint32_t side = __ballot_sync(kFull, (__float_as_uint(v[u]) >> 31) != 0u);
+      if (w0 + u * warps < nwords && lane < 2) words[w0 + u * warps + (lane ? nwords : 0)] = lane ? side : in;
+    }
   }
 }
 
+// A coordinate i from its signs: its first kF cells by their bits, the later rows from the table
+// while it is undecided, and its full median when it does not settle.  Returns the estimate or
+// marker.
 template <int R>
+__device__ __forceinline__ float resolve(const QueryParams& prm, const uint32_t* sbits, uint32_t i, uint32_t pk) {
+  constexpr int kF = R / 2 + 1;
+  const uint32_t per_row = prm.c / 32;
+  uint32_t cell[kF];  // bucket of each of the first kF rows, sign bit of the cell in bit 31
+  int lt = 0, gt = 0, rows = kF;
+#pragma unroll
+  for (int j = 0; j < kF; ++j) {
+    const uint32_t x = rot_at_lo(prm.h8.a[j], prm.h8.b[j], i), y = rot_at_lo(prm.h8.a2[j], prm.h8.b2[j], i);
+    const uint32_t w = j * per_row + ((x >> 8) & (per_row - 1u));  // place (x >> 3) mod c
+    const uint32_t in = __funnelshift_r(sbits[w], 0u, x >> 3) & 1u;
+    const uint32_t below = (__funnelshift_r(sbits[kF * per_row + w], 0u, x >> 3) ^ ~(y >> 3)) & 1u;
+    lt += (int)(in | below);
+    gt += (int)(in | (below ^ 1u));
+    cell[j] = rot_bucket(x, prm.cmask) | rot_signbit(y);
+  }
+  bool done = pk != 0u && lt >= kF && gt >= kF;
+  float v[R];
+#pragma unroll
+  for (int j = kF; j < R; ++j) {
+    v[j] = 0.f;
+    if (!done) {
+      v[j] = signed_cell(prm, j, i);
+      tally(v[j], pk, lt, gt);
+      ++rows;
+    }
+    if (j + 1 < R) done = done || (pk != 0u && lt >= kF && gt >= kF);
+  }
+  if (done) return __uint_as_float(pruned_marker(rows, rows - kF));
+#pragma unroll
+  for (int j = 0; j < kF; ++j)
+    v[j] = apply_sign(__ldg(prm.T + (size_t)j * prm.c + (cell[j] & 0x7FFFFFFFu)), cell[j] & 0x80000000u);
+  return median_of<R>(v);
+}
+
+// HM: HEAVYMIX mode (prm.keys set): each coordinate's composite key is stored and histogrammed.
+template <int R, bool HM>
 __global__ void __launch_bounds__(kBitsBlock, 1) k_query_bits(const __grid_constant__ QueryParams prm,
-                                                              const uint32_t* __restrict__ words) {
+                                                              const uint32_t* __restrict__ words,
+                                                              const __grid_constant__ GridSteps steps) {
   grid_begin();
   extern __shared__ uint4 sbits4[];
   const uint32_t* sbits = reinterpret_cast<const uint32_t*>(sbits4);
   __shared__ uint32_t sh[kBins];
+  __shared__ uint32_t queues[kBitsBlock / 32][kQueue];
   constexpr int kF = R / 2 + 1;
+  constexpr bool kNextRow = kF + 1 < R;  // a marker names fewer than R rows
+  const uint32_t per_row = prm.c / 32;
   {
-    const int64_t n4 = (int64_t)kF * (prm.c / 16) / 4;
+    const int64_t n4 = (int64_t)kF * per_row * 2 / 4;
     const uint4* src = reinterpret_cast<const uint4*>(words);
     for (int64_t w = threadIdx.x; w < n4; w += blockDim.x) sbits4[w] = __ldcg(src + w);
   }
@@ -454,91 +579,134 @@ __global__ void __launch_bounds__(kBitsBlock, 1) k_query_bits(const __grid_const
   const int64_t d = prm.d, nq = (d + 3) / 4;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int lane = threadIdx.x & 31;
+  const uint32_t below = (1u << lane) - 1u;
   const uint32_t pk = prune_key_of(prm);
-  for (int64_t q0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); q0 < nq; q0 += stride) {
+  const double theta = HM ? __ldcg(prm.theta) : 0.0;
+  const float settled = __uint_as_float(pruned_marker(kF, 0));
+  uint32_t* queue = queues[threadIdx.x >> 5];
+  uint32_t n2 = 0, n3 = 0;  // entries in the queues, the same in every lane of the warp
+  uint32_t zeros = 0;       // this lane's markers: keys of bin 0
+  const auto push3 = [&](bool who, uint32_t i) {
+    const uint32_t m = __ballot_sync(kFull, who);
+    n3 += __popc(m);
+    if (who) queue[kQueue - n3 + __popc(m & below)] = i;
+  };
+  // the estimate or marker m of coordinate i, and its key in HEAVYMIX
+  const auto record = [&](uint32_t i, float m) {
+    prm.est[i] = m;
+    const bool marker = is_pruned(__float_as_uint(m));
+    if (HM) {
+      const uint32_t key = heavy_key(marker ? 0.f : m, theta, prm.fill_seed, (uint64_t)i);
+      prm.keys[i] = key;
+      return key >> kL1Shift;
+    }
+    zeros += marker ? 1u : 0u;
+    return marker ? kNone : key_of(m) >> kL1Shift;
+  };
+  const auto drain3 = [&](bool active) {
+    uint32_t bin = kNone;
+    if (active) {
+      const uint32_t i = queue[kQueue - n3 + lane];
+      bin = record(i, resolve<R>(prm, sbits, i, pk));
+    }
+    hist_add(sh, bin);
+  };
+  const auto drain2 = [&](bool active) {
+    uint32_t i = 0;
+    bool open = false;
+    if (active) {
+      i = queue[n2 + lane];
+      const uint32_t x = rot_at_lo(prm.h8.a[kF], prm.h8.b[kF], i);
+      open = key_of(__ldg(prm.T + (size_t)kF * prm.c + rot_bucket(x, prm.cmask))) >= pk;
+      if (!open) {
+        const uint32_t bin = record(i, __uint_as_float(pruned_marker(kF + 1, 1)));
+        if (HM) atomicAdd(&sh[bin], 1u);
+      }
+    }
+    __syncwarp();  // the entries are read before the queue grows again
+    push3(open, i);
+  };
+  int64_t q0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31);
+  Rot x[kF];  // the first coordinate of the lane's quad
+#pragma unroll
+  for (int j = 0; j < kF; ++j) x[j] = rot_at(prm.h8.a[j], prm.h8.b[j], (uint32_t)((q0 + lane) * 4));
+  for (; q0 < nq; q0 += stride) {
     const int64_t q = q0 + lane;
     const int64_t i0 = q * 4;
     const int tmax = q < nq ? (d - i0 < 4 ? (int)(d - i0) : 4) : 0;
-    float m[4] = {0.f, 0.f, 0.f, 0.f};
-    if (tmax > 0) {
-      float v[4][R];
-      uint32_t cell[4][kF];  // bucket of each of the first kF rows, sign bit of the cell in bit 31
-      int lt[4], gt[4], rows[4];
-      bool done[4];
-      uint32_t count[4] = {0u, 0u, 0u, 0u};
-      // the first kF rows: classes from shared memory, no table reads
+    // bit 0: none, at most one of the rows so far has its cell outside
+    uint32_t none[4] = {1u, 1u, 1u, 1u}, one[4] = {1u, 1u, 1u, 1u};
 #pragma unroll
-      for (int j = 0; j < kF; ++j) {
-        uint64_t x = affine61_nb(prm.h.a[j], prm.h.b[j], (uint32_t)i0);
-        uint64_t y = affine61_nb(prm.h.a2[j], prm.h.b2[j], (uint32_t)i0);
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          cell[t][j] = 0u;
-          if (t < tmax) {
-            const uint32_t b = (uint32_t)x & prm.cmask;
-            const uint32_t g = (uint32_t)j * prm.c + b;
-            const uint32_t cls = (sbits[g >> 4] >> ((g & 15u) * 2u)) & 3u;
-            // a negative sign swaps the two bits; count[t] holds below-t in bits 0-7 and
-            // above-(-t) in bits 8-15: (cls * 0x201) >> 1 puts bit 1 at 0 and bit 0 at 8,
-            // cls * 0x81 puts bit 0 at 0 and bit 1 at 8
-            const uint32_t s = (uint32_t)y & 1u;
-            count[t] += ((cls * (s ? 0x81u : 0x201u)) >> (1u - s)) & 0x101u;
-            cell[t][j] = b | signbit_of(y);
-            x = step61_nb(x, prm.h.a[j]);
-            y = step61_nb(y, prm.h.a2[j]);
-          }
-        }
-      }
+    for (int j = 0; j < kF; ++j) {
+      const uint32_t* row = sbits + j * per_row;
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
-        lt[t] = (int)(count[t] & 0xFFu);
-        gt[t] = (int)(count[t] >> 8);
-        rows[t] = kF;
-        done[t] = pk != 0u && lt[t] >= kF && gt[t] >= kF;
+        // the bit of place (n8 >> 3) mod c; the shift takes its amount modulo 32
+        const uint32_t n8 = quad_lo(x[j], prm.qa[j], t);
+        const uint32_t in = __funnelshift_r(row[(n8 >> 8) & (per_row - 1u)], 0u, n8 >> 3);
+        if (kNextRow) one[t] = (one[t] & in) | none[t];
+        none[t] &= in;
       }
-      // the later rows, each only while the coordinate is undecided (read from the table)
-#pragma unroll
-      for (int j = kF; j < R; ++j) {
-        uint64_t x = affine61_nb(prm.h.a[j], prm.h.b[j], (uint32_t)i0);
-        uint64_t y = affine61_nb(prm.h.a2[j], prm.h.b2[j], (uint32_t)i0);
-        const float* row = prm.T + (size_t)j * prm.c;
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          v[t][j] = 0.f;
-          if (t < tmax) {
-            if (!done[t]) {
-              v[t][j] = apply_sign(__ldg(row + ((uint32_t)x & prm.cmask)), signbit_of(y));
-              tally(v[t][j], pk, lt[t], gt[t]);
-              ++rows[t];
-            }
-            x = step61_nb(x, prm.h.a[j]);
-            y = step61_nb(y, prm.h.a2[j]);
-          }
-        }
-        if (j + 1 < R) {
-#pragma unroll
-          for (int t = 0; t < 4; ++t) done[t] = done[t] || (pk != 0u && lt[t] >= kF && gt[t] >= kF);
-        }
-      }
-      // a coordinate that did not settle needs its full median: read its first kF cells now
-#pragma unroll
-      for (int j = 0; j < kF; ++j) {
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          v[t][j] = 0.f;
-          if (t < tmax && !done[t])
-            v[t][j] = apply_sign(__ldg(prm.T + (size_t)j * prm.c + (cell[t][j] & 0x7FFFFFFFu)),
-                                 cell[t][j] & 0x80000000u);
-        }
-      }
-#pragma unroll
-      for (int t = 0; t < 4; ++t)
-        m[t] = done[t] ? __uint_as_float(pruned_marker(rows[t], rows[t] - kF)) : median_of<R>(v[t]);
-      store_est(prm, i0, tmax, m);
+      x[j] = rot_add(x[j], steps.a[j]);
     }
+    uint32_t hk[4];
+    if (tmax > 0) {
+      const float m[4] = {settled, settled, settled, settled};
+      store_est(prm, i0, tmax, m);
+      if (HM) {  // the keys of the settled; those of the queued are replaced below
 #pragma unroll
-    for (int t = 0; t < 4; ++t) hist_add(sh, t < tmax ? (key_of(m[t]) >> kL1Shift) : kNone);
+        for (int t = 0; t < 4; ++t) hk[t] = heavy_key(0.f, theta, prm.fill_seed, (uint64_t)(i0 + t));
+        if (tmax == 4) {
+          *reinterpret_cast<uint4*>(prm.keys + i0) = make_uint4(hk[0], hk[1], hk[2], hk[3]);
+        } else {
+          for (int t = 0; t < tmax; ++t) prm.keys[i0 + t] = hk[t];
+        }
+      }
+    }
+    zeros += (uint32_t)tmax;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const bool open = t < tmax && !(none[t] & 1u);
+      const bool second = kNextRow && open && (one[t] & 1u);
+      if (HM) {
+        if (t < tmax && !open) atomicAdd(&sh[hk[t] >> kL1Shift], 1u);  // spread over 1024 bins
+      } else if (open) {
+        --zeros;
+      }
+      if (kNextRow) {
+        const uint32_t who = __ballot_sync(kFull, second);
+        if (second) queue[n2 + __popc(who & below)] = (uint32_t)i0 + t;
+        n2 += __popc(who);
+      }
+      push3(open && !second, (uint32_t)i0 + t);
+    }
+    __syncwarp();  // the queues, and the markers that the estimates below replace
+    while (true) {
+      while (n3 >= 32) {
+        drain3(true);
+        n3 -= 32;
+      }
+      if (!kNextRow || n2 < 32) break;
+      n2 -= 32;
+      drain2(true);
+      __syncwarp();
+    }
+    __syncwarp();
   }
+  if (kNextRow) {
+    const uint32_t n = n2;
+    n2 = 0;
+    drain2((uint32_t)lane < n);
+    __syncwarp();
+  }
+  while (n3 > 0) {
+    const uint32_t n = n3 < 32 ? n3 : 32;
+    drain3((uint32_t)lane < n);
+    n3 -= n;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) zeros += __shfl_down_sync(kFull, zeros, o);
+  if (!HM && lane == 0 && zeros) atomicAdd(&sh[0], zeros);
   hist_flush(sh, prm.hist, kBins);
   last_block_pick(prm.hist, 11, prm.st, 0, prm.k);
 }
@@ -568,11 +736,7 @@ __global__ void __launch_bounds__(kBlock) k_repair(const __grid_constant__ Query
       if (is_pruned(__float_as_uint(e))) {
         float v[R];
 #pragma unroll
-        for (int j = 0; j < R; ++j) {
-          const uint64_t x = affine61(prm.h.a[j], prm.h.b[j], (uint32_t)i);
-          const uint64_t y = affine61(prm.h.a2[j], prm.h.b2[j], (uint32_t)i);
-          v[j] = apply_sign(__ldg(prm.T + (size_t)j * prm.c + ((uint32_t)x & prm.cmask)), signbit_of(y));
-        }
+        for (int j = 0; j < R; ++j) v[j] = signed_cell(prm, j, (uint32_t)i);
         e = median_of<R>(v);
         prm.est[i] = e;
       }
@@ -1235,15 +1399,17 @@ constexpr QueryLauncher QueryTable<Rs...>::table[sizeof...(Rs)];
 template <int R>
 cudaError_t launch_query_bits_r(const QueryParams& p, uint32_t* words, cudaStream_t s) {
   constexpr int kF = R / 2 + 1;
-  const int64_t nwords = (int64_t)kF * (p.c / 16);
-  const int gw = (int)((nwords + kBlock - 1) / kBlock);
-  launch(k_pbits, gw, kBlock, s, p.T, nwords, p.st, words);
-  auto kern = k_query_bits<R>;
-  const size_t smem = (size_t)nwords * sizeof(uint32_t);
+  const int64_t nwords = (int64_t)kF * (p.c / 32);  // words of one kind of bit
+  const int64_t warps = (nwords + kBlock / 32 - 1) / (kBlock / 32), cap = (int64_t)device_info().sms * 8;
+  launch(k_pbits, (int)(warps < cap ? warps : cap), kBlock, s, p.T, p.c, nwords, p.st, words);
+  auto kern = p.keys ? k_query_bits<R, true> : k_query_bits<R, false>;
+  const size_t smem = (size_t)nwords * 2 * sizeof(uint32_t);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int64_t need = ((p.d + 3) / 4 + kBitsBlock - 1) / kBitsBlock;
   const int grid = (int)(need < device_info().sms ? (need < 1 ? 1 : need) : device_info().sms);
+  GridSteps steps = {};
+  for (int j = 0; j < kF; ++j) steps.a[j] = 8 * mulmod61(p.h.a[j], (uint64_t)grid * kBitsBlock * 4);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(kBitsBlock);
@@ -1254,7 +1420,7 @@ cudaError_t launch_query_bits_r(const QueryParams& p, uint32_t* words, cudaStrea
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, kern, p, (const uint32_t*)words);
+  e = cudaLaunchKernelEx(&cfg, kern, p, (const uint32_t*)words, steps);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -1372,6 +1538,15 @@ QueryParams make_query_params(const float* merged, const HashCoeffs& h, int r, u
   qp.theta = nullptr;
   qp.fill_seed = 0;
   qp.h = h;
+  std::memset(&qp.h8, 0, sizeof(qp.h8));
+  std::memset(qp.qa, 0, sizeof(qp.qa));
+  for (int j = 0; j < r; ++j) {
+    qp.h8.a[j] = 8 * h.a[j];
+    qp.h8.b[j] = 8 * h.b[j];
+    qp.h8.a2[j] = 8 * h.a2[j];
+    qp.h8.b2[j] = 8 * h.b2[j];
+    for (uint64_t t = 1; t <= 3 && j < GS_MAX_ROWS / 2 + 1; ++t) qp.qa[j][t - 1] = 8 * mulmod61(h.a[j], t);
+  }
   return qp;
 }
 
@@ -1436,6 +1611,13 @@ cudaError_t clear_selection(const Workspace& w, cudaStream_t s) {
   return err;
 }
 
+// The pruning query by k_query_bits; its words go in the candidate area, which the selection only
+// uses after the query.
+cudaError_t launch_query_bits(const QueryParams& p, const Workspace& w, cudaStream_t s) {
+  using T = BitsTable<1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16>;
+  return T::table[p.r - 1](p, reinterpret_cast<uint32_t*>(w.cand), s);
+}
+
 // Levels 2 and 3 and the ordered output, after the level-1 histogram and pick of `src` keys.
 cudaError_t select_from_keys(const Workspace& w, const float* src, int vec, uint32_t kmask, int64_t d, int64_t k,
                              int64_t* idx_out, cudaStream_t s) {
@@ -1475,9 +1657,7 @@ cudaError_t launch_query_topk(const float* merged, const HashCoeffs& h, int r, u
     if ((err = T::table[r - 1](qp, w.hist + 4 * kBins, j_target, s)) != cudaSuccess) return err;
   }
   if (qp.prune && query_uses_bits(r, c)) {
-    // the classes go in the candidate area, which the selection only uses after the query
-    using T = BitsTable<1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16>;
-    if ((err = T::table[r - 1](qp, reinterpret_cast<uint32_t*>(w.cand), s)) != cudaSuccess) return err;
+    if ((err = launch_query_bits(qp, w, s)) != cudaSuccess) return err;
   } else if ((err = launch_query(qp, s)) != cudaSuccess) {
     return err;
   }
@@ -1528,7 +1708,9 @@ cudaError_t launch_query_heavymix(const float* merged, const HashCoeffs& h, int 
   qp.keys = keys;
   qp.theta = theta;
   qp.fill_seed = fill_seed;
-  if ((err = launch_query(qp, s)) != cudaSuccess) return err;
+  if (prune && query_uses_bits(r, c)) err = launch_query_bits(qp, w, s);
+  else err = launch_query(qp, s);
+  if (err != cudaSuccess) return err;
   if ((err = mark(marks, 1, s)) != cudaSuccess) return err;
   if ((err = select_from_keys(w, reinterpret_cast<const float*>(keys), 1, 0xFFFFFFFFu, d, k, idx_out, s)) !=
       cudaSuccess)
