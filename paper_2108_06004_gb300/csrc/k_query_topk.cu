@@ -33,12 +33,15 @@
 #include <cstring>
 #include <mutex>
 
+#include <cooperative_groups.h>
 #include <cuda.h>
 
 #include "chain_plan.h"
 #include "gs_common.cuh"
 
 namespace gs {
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -283,7 +286,7 @@ struct QueryParams {
   int32_t r;
   uint32_t c, cmask;
   int32_t vec;        // est 16-byte aligned
-  int32_t hist_on;    // build the level-1 histogram of |est| keys and pick
+  int32_t pick;       // the last CTA picks the level-1 bin from the histogram of the keys
   int32_t prune;      // skip rows below st->prune_key (estimate internal to the workspace)
   uint32_t* keys;     // HEAVYMIX: also store each coordinate's composite key here, and build the
                       // level-1 histogram (and pick) on those keys instead of |est|
@@ -445,16 +448,12 @@ __global__ void __launch_bounds__(kBlock, R <= 7 ? 4 : 1) k_query(const __grid_c
         }
       }
     }
-    if (prm.hist_on) {
 #pragma unroll
-      for (int t = 0; t < 4; ++t)
-        hist_add(sh, t < tmax ? ((HM ? hk[t] : key_of(m[t])) >> kL1Shift) : kNone);
-    }
+    for (int t = 0; t < 4; ++t)
+      hist_add(sh, t < tmax ? ((HM ? hk[t] : key_of(m[t])) >> kL1Shift) : kNone);
   }
-  if (prm.hist_on) {
-    hist_flush(sh, prm.hist, kBins);
-    last_block_pick(prm.hist, 11, prm.st, 0, prm.k);
-  }
+  hist_flush(sh, prm.hist, kBins);
+  if (prm.pick) last_block_pick(prm.hist, 11, prm.st, 0, prm.k);
 }
 
 // ---- the pruning query with the first rows classified in shared memory ---------------------
@@ -899,12 +898,10 @@ __global__ void __launch_bounds__(kBlock) k_query_generic(const __grid_constant_
       }
       bin = key >> kL1Shift;
     }
-    if (prm.hist_on) hist_add(sh, bin);
+    hist_add(sh, bin);
   }
-  if (prm.hist_on) {
-    hist_flush(sh, prm.hist, kBins);
-    last_block_pick(prm.hist, 11, prm.st, 0, prm.k);
-  }
+  hist_flush(sh, prm.hist, kBins);
+  if (prm.pick) last_block_pick(prm.hist, 11, prm.st, 0, prm.k);
 }
 
 // Four float4 of est per thread in flight (kU strides of the grid-stride loop).
@@ -1137,6 +1134,217 @@ __global__ void __launch_bounds__(kBmThreads) k_bm_write(const uint32_t* __restr
       }
       if (take) {
         if ((int64_t)pos < k) idx_out[pos] = (w0 + j) * 32 + b;
+        ++pos;
+      }
+    }
+  }
+}
+
+// ---- selection by one cluster ----------------------------------------------------------------
+// For short vectors the selection's six kernels and their picks are almost all latency (33 us of a
+// 92 us step at d = 2^20).  Here one cluster of 16 CTAs, the widest there is, does levels 2 and 3 and
+// the ordered output in a single launch: each CTA owns a contiguous run of coordinates and keeps its
+// bitmaps and candidates in shared memory; the histograms meet in the first CTA's shared memory, and
+// cluster barriers stand where the kernels were.  Query and selection in us, k = d/1000 (d/100), six
+// kernels / one cluster: d = 100k 35.2 / 22.0 (37.1 / 22.1), 300k 39.1 / 25.9 (42.4 / 28.2), 2^20 50.1 / 39.7
+// (53.7 / 47.2), 2M 68.6 / 64.4 (72.2 / 75.7), 4M 108 / 112 (113 / 171): beyond 1.5 * 2^20 the 136 idle SMs
+// cost more than the launches.
+constexpr int kSmallCtas = 16;
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallList = 16384;                   // candidates kept per CTA
+constexpr int64_t kSmallMaxDim = int64_t(3) << 19;  // 3072 bitmap words per CTA
+
+bool selects_small(int64_t d) { return d <= kSmallMaxDim; }
+
+struct SmallShared {
+  uint32_t h2[kBins];
+  uint32_t h3[1 << kL3Bits];
+  uint32_t sum[kBins];       // a histogram of the whole cluster
+  uint2 list[kSmallList];    // candidates (index, key) of this CTA
+  uint32_t n;                // how many there are (the list may hold fewer)
+  uint32_t bin, rem;         // a pick
+  uint32_t gt, eq;           // this CTA's keys above and equal to tau
+};
+
+// The bin of sum[0..nbins) that holds the k_rem-th largest key, and what is still to take in it.
+__device__ __forceinline__ void pick_shared(SmallShared& sm, int nbins, uint32_t k_rem) {
+  const int per = nbins / kSmallThreads;  // 1 or 2
+  const int r0 = threadIdx.x * per;       // positions counted from the top bin
+  uint32_t cnt[2] = {0u, 0u};
+  for (int t = 0; t < per; ++t) cnt[t] = sm.sum[nbins - 1 - (r0 + t)];
+  uint32_t total;
+  uint32_t cum = block_excl_scan(cnt[0] + cnt[1], &total);
+  for (int t = 0; t < per; ++t) {
+    if (cum < k_rem && cum + cnt[t] >= k_rem) {
+      sm.bin = (uint32_t)(nbins - 1 - (r0 + t));
+      sm.rem = k_rem - cum;
+    }
+    cum += cnt[t];
+  }
+  __syncthreads();
+}
+
+// Calls f(index, key) for every coordinate of [c0, c1), c0 a multiple of 4.
+template <typename F>
+__device__ __forceinline__ void for_keys(const float* __restrict__ src, int64_t c0, int64_t c1, int vec, uint32_t kmask,
+                                         const F& f) {
+  for (int64_t b = c0; b < c1; b += 4 * kU * kSmallThreads) {
+    float v[kU][4];
+    int tm[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int64_t i0 = b + 4 * ((int64_t)u * kSmallThreads + threadIdx.x);
+      tm[u] = i0 < c1 ? (c1 - i0 < 4 ? (int)(c1 - i0) : 4) : 0;
+      if (vec && tm[u] == 4) {
+        const float4 x = __ldcg(reinterpret_cast<const float4*>(src + i0));
+        v[u][0] = x.x; v[u][1] = x.y; v[u][2] = x.z; v[u][3] = x.w;
+      } else {
+#pragma unroll
+        for (int t = 0; t < 4; ++t) v[u][t] = t < tm[u] ? __ldcg(src + i0 + t) : 0.f;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int64_t i0 = b + 4 * ((int64_t)u * kSmallThreads + threadIdx.x);
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (t < tm[u]) f((uint32_t)i0 + t, __float_as_uint(v[u][t]) & kmask);
+    }
+  }
+}
+
+// picked: level 1 was picked already (st); otherwise it is picked from hist1 here, by every CTA.
+__global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThreads, 1)
+    k_select_small(const float* __restrict__ src, int64_t d, int vec, uint32_t kmask, const uint32_t* __restrict__ hist1,
+                   const SelectState* st, int picked, uint32_t k, int64_t* __restrict__ idx_out) {
+  grid_begin();
+  extern __shared__ uint4 small_dyn[];
+  SmallShared& sm = *reinterpret_cast<SmallShared*>(small_dyn);
+  cg::cluster_group cluster = cg::this_cluster();
+  const uint32_t rank = cluster.block_rank();
+  const int64_t nbw = (d + 31) / 32;
+  const int64_t per = (nbw + kSmallCtas - 1) / kSmallCtas;  // bitmap words of a CTA
+  uint32_t* gt_bm = reinterpret_cast<uint32_t*>(small_dyn) + sizeof(SmallShared) / sizeof(uint32_t);
+  uint32_t* eq_bm = gt_bm + per;
+  const int64_t w0 = (int64_t)rank * per;
+  const int nw = (int)(w0 >= nbw ? 0 : (nbw - w0 < per ? nbw - w0 : per));
+  const int64_t c0 = w0 * 32, c1 = c0 + (int64_t)nw * 32 < d ? c0 + (int64_t)nw * 32 : d;
+
+  for (int b = threadIdx.x; b < kBins; b += kSmallThreads) {
+    sm.h2[b] = 0;
+    sm.sum[b] = picked ? 0u : __ldcg(&hist1[b]);
+  }
+  for (int b = threadIdx.x; b < (1 << kL3Bits); b += kSmallThreads) sm.h3[b] = 0;
+  for (int w = threadIdx.x; w < 2 * (int)per; w += kSmallThreads) gt_bm[w] = 0;  // both bitmaps
+  if (threadIdx.x == 0) {
+    sm.n = 0;
+    if (picked) {
+      sm.bin = __ldcg(&st->prefix);
+      sm.rem = __ldcg(&st->k_rem);
+    }
+  }
+  __syncthreads();
+  if (!picked) pick_shared(sm, kBins, k);
+  const uint32_t b1 = sm.bin, k1 = sm.rem;
+  cluster.sync();  // every histogram is clear
+
+  // level 2: keys above the bin are taken, those in it are candidates
+  for_keys(src, c0, c1, vec, kmask, [&](uint32_t i, uint32_t key) {
+    if ((key >> kL1Shift) < b1) return;
+    if ((key >> kL1Shift) > b1) {
+      const uint32_t at = i - (uint32_t)c0;
+      atomicOr(&gt_bm[at >> 5], 1u << (at & 31));
+      return;
+    }
+    atomicAdd(&sm.h2[(key >> kL2Shift) & (kBins - 1)], 1u);
+    const uint32_t am = __activemask();
+    const int lane = threadIdx.x & 31, leader = __ffs(am) - 1;
+    uint32_t slot = 0;
+    if (lane == leader) slot = atomicAdd(&sm.n, (uint32_t)__popc(am));
+    slot = __shfl_sync(am, slot, leader) + __popc(am & ((1u << lane) - 1u));
+    if (slot < (uint32_t)kSmallList) sm.list[slot] = make_uint2(i, key);
+  });
+  __syncthreads();
+  const uint32_t n = sm.n;
+  uint32_t* const total2 = cluster.map_shared_rank(sm.h2, 0);
+  if (rank != 0)
+    for (int b = threadIdx.x; b < kBins; b += kSmallThreads)
+      if (sm.h2[b]) atomicAdd(&total2[b], sm.h2[b]);
+  cluster.sync();
+  for (int b = threadIdx.x; b < kBins; b += kSmallThreads) sm.sum[b] = total2[b];
+  __syncthreads();
+  pick_shared(sm, kBins, k1);
+  const uint32_t p22 = (b1 << 11) | sm.bin, k2 = sm.rem;
+
+  // level 3, over the candidates (the keys again where they overflow the list)
+  const auto candidates = [&](const auto& f) {
+    if (n <= (uint32_t)kSmallList) {
+      for (uint32_t t = threadIdx.x; t < n; t += kSmallThreads) f(sm.list[t].x, sm.list[t].y);
+    } else {
+      for_keys(src, c0, c1, vec, kmask, [&](uint32_t i, uint32_t key) {
+        if ((key >> kL1Shift) == b1) f(i, key);
+      });
+    }
+  };
+  candidates([&](uint32_t, uint32_t key) {
+    if ((key >> kL2Shift) == p22) atomicAdd(&sm.h3[key & ((1u << kL3Bits) - 1u)], 1u);
+  });
+  __syncthreads();
+  uint32_t* const total3 = cluster.map_shared_rank(sm.h3, 0);
+  if (rank != 0)
+    for (int b = threadIdx.x; b < (1 << kL3Bits); b += kSmallThreads)
+      if (sm.h3[b]) atomicAdd(&total3[b], sm.h3[b]);
+  cluster.sync();
+  for (int b = threadIdx.x; b < (1 << kL3Bits); b += kSmallThreads) sm.sum[b] = total3[b];
+  __syncthreads();
+  pick_shared(sm, 1 << kL3Bits, k2);
+  const uint32_t tau = (p22 << kL3Bits) | sm.bin, need_eq = sm.rem;
+
+  candidates([&](uint32_t i, uint32_t key) {
+    const uint32_t at = i - (uint32_t)c0;
+    if (key > tau) atomicOr(&gt_bm[at >> 5], 1u << (at & 31));
+    else if (key == tau) atomicOr(&eq_bm[at >> 5], 1u << (at & 31));
+  });
+  __syncthreads();
+
+  // ordered output: this CTA's counts, those of the CTAs before it, then as in k_bm_write
+  const int each = (nw + kSmallThreads - 1) / kSmallThreads;  // words of a thread
+  const int t0 = threadIdx.x * each, t1 = t0 + each < nw ? t0 + each : nw;
+  uint32_t gt = 0, eq = 0;
+  for (int w = t0; w < t1; ++w) {
+    gt += __popc(gt_bm[w]);
+    eq += __popc(eq_bm[w]);
+  }
+  uint32_t all_gt, all_eq;
+  const uint32_t pre_gt = block_excl_scan(gt, &all_gt), pre_eq = block_excl_scan(eq, &all_eq);
+  if (threadIdx.x == 0) {
+    sm.gt = all_gt;
+    sm.eq = all_eq;
+  }
+  cluster.sync();
+  uint32_t base = 0, eqx = 0;
+  for (uint32_t c = 0; c < rank; ++c) {
+    base += *cluster.map_shared_rank(&sm.gt, c);
+    eqx += *cluster.map_shared_rank(&sm.eq, c);
+  }
+  base += eqx < need_eq ? eqx : need_eq;
+  cluster.sync();  // no CTA leaves while others read its shared memory
+  if (gt + eq == 0) return;
+  const uint32_t eq_quota = need_eq > eqx ? need_eq - eqx : 0u;
+  uint32_t pos = base + pre_gt + (pre_eq < eq_quota ? pre_eq : eq_quota);
+  uint32_t eq_rank = pre_eq;
+  for (int w = t0; w < t1; ++w) {
+    uint32_t bits = gt_bm[w] | eq_bm[w];
+    while (bits) {
+      const int b = __ffs(bits) - 1;
+      bits &= bits - 1u;
+      bool take = (gt_bm[w] >> b) & 1u;
+      if (!take) {
+        take = eq_rank < eq_quota;
+        ++eq_rank;
+      }
+      if (take) {
+        if (pos < k) idx_out[pos] = c0 + (int64_t)w * 32 + b;
         ++pos;
       }
     }
@@ -1532,7 +1740,7 @@ QueryParams make_query_params(const float* merged, const HashCoeffs& h, int r, u
   qp.c = c;
   qp.cmask = c - 1;
   qp.vec = (reinterpret_cast<uintptr_t>(est) & 15u) == 0 ? 1 : 0;
-  qp.hist_on = 1;
+  qp.pick = 1;
   qp.prune = 0;
   qp.keys = nullptr;
   qp.theta = nullptr;
@@ -1601,12 +1809,12 @@ cudaError_t mark(const cudaEvent_t* marks, int i, cudaStream_t s) {
   return (marks && marks[i]) ? cudaEventRecordWithFlags(marks[i], s, cudaEventRecordExternal) : cudaSuccess;
 }
 
-// Histograms, state and both bitmaps back to zero.
-cudaError_t clear_selection(const Workspace& w, cudaStream_t s) {
-  cudaError_t err = cudaMemsetAsync(w.hist, 0, 5 * kBins * sizeof(uint32_t), s);
-  if (err == cudaSuccess) err = cudaMemsetAsync(w.st, 0, sizeof(SelectState), s);
-  // the two bitmaps are adjacent: clear both at once
-  if (err == cudaSuccess)
+// Histograms and state (adjacent) and, unless the selection goes by one cluster, both bitmaps
+// (adjacent) back to zero.
+cudaError_t clear_selection(const Workspace& w, int64_t d, cudaStream_t s) {
+  const size_t head = (size_t)(reinterpret_cast<char*>(w.st + 1) - reinterpret_cast<char*>(w.hist));
+  cudaError_t err = cudaMemsetAsync(w.hist, 0, head, s);
+  if (err == cudaSuccess && !selects_small(d))
     err = cudaMemsetAsync(w.gt_bm, 0, (size_t)(reinterpret_cast<char*>(w.blk) - reinterpret_cast<char*>(w.gt_bm)), s);
   return err;
 }
@@ -1616,6 +1824,28 @@ cudaError_t clear_selection(const Workspace& w, cudaStream_t s) {
 cudaError_t launch_query_bits(const QueryParams& p, const Workspace& w, cudaStream_t s) {
   using T = BitsTable<1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16>;
   return T::table[p.r - 1](p, reinterpret_cast<uint32_t*>(w.cand), s);
+}
+
+// Levels 2 and 3 and the ordered output by one cluster; `picked`: see k_select_small.
+cudaError_t select_small(const float* src, int vec, uint32_t kmask, const uint32_t* hist1, const SelectState* st,
+                         int picked, int64_t d, int64_t k, int64_t* idx_out, cudaStream_t s) {
+  const int64_t per = ((d + 31) / 32 + kSmallCtas - 1) / kSmallCtas;
+  const size_t smem = sizeof(SmallShared) + 2 * (size_t)per * sizeof(uint32_t);
+  cudaError_t e = cudaFuncSetAttribute(k_select_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_select_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kSmallCtas);
+  cfg.blockDim = dim3(kSmallThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  e = cudaLaunchKernelEx(&cfg, k_select_small, src, d, vec, kmask, hist1, st, picked, (uint32_t)k, idx_out);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // Levels 2 and 3 and the ordered output, after the level-1 histogram and pick of `src` keys.
@@ -1644,7 +1874,7 @@ cudaError_t launch_query_topk(const float* merged, const HashCoeffs& h, int r, u
                               void* workspace, cudaStream_t s, const cudaEvent_t* marks) {
   Workspace w = carve(workspace, d);
   float* est = est_out ? est_out : w.est;
-  cudaError_t err = clear_selection(w, s);
+  cudaError_t err = clear_selection(w, d, s);
   if (err != cudaSuccess) return err;
   if ((err = mark(marks, 0, s)) != cudaSuccess) return err;
 
@@ -1652,6 +1882,7 @@ cudaError_t launch_query_topk(const float* merged, const HashCoeffs& h, int r, u
   // rows are pruned only while the estimate stays internal: a caller's est_out gets every value
   const uint32_t j_target = sample_rank(d, k);
   qp.prune = (!est_out && can_prune(r, c, d) && j_target > 0) ? 1 : 0;
+  qp.pick = (qp.prune || !selects_small(d)) ? 1 : 0;  // k_repair needs the pick, and so do many CTAs
   if (qp.prune) {
     using T = SampleTable<1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16>;
     if ((err = T::table[r - 1](qp, w.hist + 4 * kBins, j_target, s)) != cudaSuccess) return err;
@@ -1666,8 +1897,9 @@ cudaError_t launch_query_topk(const float* merged, const HashCoeffs& h, int r, u
     if ((err = T::table[r - 1](qp, w.hist + 3 * kBins, s)) != cudaSuccess) return err;
   }
   if ((err = mark(marks, 1, s)) != cudaSuccess) return err;
-  if ((err = select_from_keys(w, est, qp.vec, 0x7FFFFFFFu, d, k, idx_out, s)) != cudaSuccess) return err;
-  return mark(marks, 2, s);
+  if (selects_small(d)) err = select_small(est, qp.vec, 0x7FFFFFFFu, w.hist, w.st, qp.pick, d, k, idx_out, s);
+  else err = select_from_keys(w, est, qp.vec, 0x7FFFFFFFu, d, k, idx_out, s);
+  return err != cudaSuccess ? err : mark(marks, 2, s);
 }
 
 cudaError_t launch_query_ceiling_probe(const float* merged, const HashCoeffs& h, int r, uint32_t c, int64_t d,
@@ -1691,7 +1923,7 @@ cudaError_t launch_query_heavymix(const float* merged, const HashCoeffs& h, int 
   double* sumsq = reinterpret_cast<double*>(extra + align256((size_t)d * sizeof(uint32_t)));
   double* theta = sumsq + GS_MAX_ROWS;
   float* est = est_out ? est_out : w.est;
-  cudaError_t err = clear_selection(w, s);
+  cudaError_t err = clear_selection(w, d, s);
   if (err == cudaSuccess) err = cudaMemsetAsync(sumsq, 0, 256, s);
   if (err == cudaSuccess) err = mark(marks, 0, s);
   if (err != cudaSuccess) return err;
@@ -1705,6 +1937,7 @@ cudaError_t launch_query_heavymix(const float* merged, const HashCoeffs& h, int 
   // the query stores each coordinate's composite key and picks on their level-1 histogram
   QueryParams qp = make_query_params(merged, h, r, c, d, k, est, w.hist, w.st);
   qp.prune = prune;
+  qp.pick = (prune || !selects_small(d)) ? 1 : 0;
   qp.keys = keys;
   qp.theta = theta;
   qp.fill_seed = fill_seed;
@@ -1712,10 +1945,10 @@ cudaError_t launch_query_heavymix(const float* merged, const HashCoeffs& h, int 
   else err = launch_query(qp, s);
   if (err != cudaSuccess) return err;
   if ((err = mark(marks, 1, s)) != cudaSuccess) return err;
-  if ((err = select_from_keys(w, reinterpret_cast<const float*>(keys), 1, 0xFFFFFFFFu, d, k, idx_out, s)) !=
-      cudaSuccess)
-    return err;
-  return mark(marks, 2, s);
+  const float* src = reinterpret_cast<const float*>(keys);
+  if (selects_small(d)) err = select_small(src, 1, 0xFFFFFFFFu, w.hist, w.st, qp.pick, d, k, idx_out, s);
+  else err = select_from_keys(w, src, 1, 0xFFFFFFFFu, d, k, idx_out, s);
+  return err != cudaSuccess ? err : mark(marks, 2, s);
 }
 
 // ---- scratch without allocation ---------------------------------------------------------
@@ -1813,12 +2046,13 @@ cudaError_t launch_query_topk_noalloc(const float* merged, const HashCoeffs& h, 
   uint32_t* blk_base = blk_eq + nseg;
   uint32_t* blk_eqx = blk_base + nseg;
   // the histograms and the state must start at zero; the segment counters are overwritten
-  err = cudaMemsetAsync(hist, 0, kNoallocHistBytes, s);
-  if (err == cudaSuccess) err = cudaMemsetAsync(st, 0, sizeof(SelectState), s);
+  err = cudaMemsetAsync(hist, 0, kNoallocHistBytes + kNoallocStateBytes, s);
   if (err != cudaSuccess) return err;
 
-  const QueryParams qp = make_query_params(merged, h, r, c, d, k, est_out, hist, st);
+  QueryParams qp = make_query_params(merged, h, r, c, d, k, est_out, hist, st);
+  qp.pick = selects_small(d) ? 0 : 1;
   if ((err = launch_query(qp, s)) != cudaSuccess) return err;
+  if (selects_small(d)) return select_small(est_out, qp.vec, 0x7FFFFFFFu, hist, st, 0, d, k, idx_out, s);
   const int hgrid = persistent_grid(k_hist, (d + 3) / 4 / kU, kBlock);
   launch(k_hist, hgrid, kBlock, s, est_out, d, qp.vec, st, hist + kBins, kL2Shift, 11, 1);
   launch(k_hist, hgrid, kBlock, s, est_out, d, qp.vec, st, hist + 2 * kBins, 0, kL3Bits, 2);
