@@ -273,6 +273,7 @@ gs_status accumulate_insert_impl(gs_sketch* sk, int32_t first, int32_t n, float*
     p.r = sk->r;
     p.c = (uint32_t)sk->c;
     p.cmask = (uint32_t)sk->c - 1;
+    p.cinv = gs::bucket_inverse((uint32_t)sk->c);
     p.rho = rho;
     p.h = sk->h;
     if (!sk->rotation.empty()) {
@@ -326,6 +327,7 @@ gs_status insert_all_impl(gs_sketch* sk, const float* const* vec, int64_t d, cud
     p.r = sk->r;
     p.c = (uint32_t)sk->c;
     p.cmask = (uint32_t)sk->c - 1;
+    p.cinv = gs::bucket_inverse((uint32_t)sk->c);
     p.h = sk->h;
     if (!sk->rotation.empty()) {
       GS_TRY(insert_chains(sk, p.table, W, W, 0, p.e, nw, d, s));
@@ -849,6 +851,7 @@ gs_status gs_sketch_insert(gs_sketch* sk, int32_t worker, const float* vec, int6
   p.j1 = sk->r;
   p.c = (uint32_t)sk->c;
   p.cmask = (uint32_t)sk->c - 1;
+  p.cinv = gs::bucket_inverse((uint32_t)sk->c);
   p.h = sk->h;
   cudaError_t e = gs::launch_insert_lane(p, W, as_stream(stream));
   if (e != cudaSuccess) return cuda_fail(e, "insert launch");
@@ -909,6 +912,7 @@ gs_status gs_accumulate_insert_staged(gs_sketch* sk, int32_t first_worker, int32
     p.r = sk->r;
     p.c = (uint32_t)sk->c;
     p.cmask = (uint32_t)sk->c - 1;
+    p.cinv = gs::bucket_inverse((uint32_t)sk->c);
     p.h = sk->h;
     p.j0 = 0;
     p.j1 = sk->r;
@@ -1417,6 +1421,7 @@ gs_status gs_insert_request_ceiling(gs_sketch* sk, int64_t d, void* window, size
     p.r = sk->r;
     p.c = (uint32_t)sk->c;
     p.cmask = (uint32_t)sk->c - 1;
+    p.cinv = gs::bucket_inverse((uint32_t)sk->c);
     p.rho = 0.9f;
     p.evict = sk->rows_per_pass < sk->r;
     p.winmask = GS_CEILING_WINDOW_FLOATS - 1;

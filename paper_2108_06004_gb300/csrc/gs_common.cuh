@@ -43,10 +43,13 @@ __device__ __forceinline__ uint64_t step61(uint64_t x, uint64_t a) {
   return x >= kP61 ? x - kP61 : x;
 }
 
+// x mod c.  For c not a power of two, with cinv = floor(2^64 / c): the estimate x * cinv >> 64 of the
+// quotient is at most 1 below it (x < 2^61), so the remainder needs one correction.
 template <bool POW2>
-__device__ __forceinline__ uint32_t bucket_of(uint64_t x, uint32_t c, uint32_t cmask) {
+__device__ __forceinline__ uint32_t bucket_of(uint64_t x, uint32_t c, uint32_t cmask, uint64_t cinv) {
   if (POW2) return (uint32_t)x & cmask;
-  return (uint32_t)(x % (uint64_t)c);
+  const uint32_t r = (uint32_t)x - (uint32_t)__umul64hi(x, cinv) * c;
+  return r >= c ? r - c : r;
 }
 
 // Sign bit (bit 31 set for s = -1): s_j(i) = -1 when the second hash value is odd.
@@ -133,6 +136,7 @@ struct InsertParams {
   int32_t r;
   int32_t j0, j1;    // rows inserted by this launch: [j0, j1)
   uint32_t c, cmask;
+  uint64_t cinv;     // bucket_inverse(c)
   float rho;
   int32_t evict;     // the table does not fit L2 beside the streams: mark these evict_first
   int64_t winmask;   // request-ceiling probe only: vector offsets are taken modulo winmask + 1
@@ -262,6 +266,7 @@ cudaError_t launch_query_topk_noalloc(const float* merged, const HashCoeffs& h, 
                                       int64_t d, int64_t k, int64_t* idx_out, float* est_out,
                                       cudaStream_t s);
 
+inline uint64_t bucket_inverse(uint32_t c) { return c > 1 ? ~0ull / c : 0; }  // floor(2^64 / c) unless c is a power of two
 inline bool is_pow2(uint32_t c) { return c && !(c & (c - 1)); }
 
 // ---- launches -----------------------------------------------------------------------

@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kBlock) k_accumulate_insert(const __grid_const
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
         if (t < tmax) {
-          const uint32_t bk = bucket_of<POW2>(x, prm.c, prm.cmask);
+          const uint32_t bk = bucket_of<POW2>(x, prm.c, prm.cmask, prm.cinv);
           const uint32_t sb = signbit_of(y);
           float* cell = row + (size_t)bk * W;
           if (W == 1) {
@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(kBlock) k_accumulate_insert_coop(const __grid_
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
         if (t < tmax) {
-          const uint32_t bk = bucket_of<POW2>(x, prm.c, prm.cmask);
+          const uint32_t bk = bucket_of<POW2>(x, prm.c, prm.cmask, prm.cinv);
           const uint32_t sb = signbit_of(y);
           red_add_v4_keep(row + (size_t)bk * W, apply_sign(ev[0][t], sb), apply_sign(ev[1][t], sb),
                           apply_sign(ev[2][t], sb), apply_sign(ev[3][t], sb), pol_table);
@@ -367,7 +367,7 @@ __global__ void __launch_bounds__(kBlock) k_insert_lane(const __grid_constant__ 
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
         if (t < tmax) {
-          const uint32_t bk = bucket_of<false>(x, prm.c, prm.cmask);
+          const uint32_t bk = bucket_of<false>(x, prm.c, prm.cmask, prm.cinv);
           red_add_f32(row + (size_t)bk * W, apply_sign(ev[t], signbit_of(y)));
           x = step61(x, a);
           y = step61(y, a2);
@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(kBlock) k_insert_staged(const __grid_constant_
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
       if (t < tmax) {
-        const uint32_t bk = bucket_of<POW2>(x, c, prm.cmask);
+        const uint32_t bk = bucket_of<POW2>(x, c, prm.cmask, prm.cinv);
         const uint32_t sb = signbit_of(y);
 #pragma unroll
         for (int w = 0; w < WT; ++w) atomicAdd(&tile[bk * WT + w], apply_sign(ev[w][t], sb));

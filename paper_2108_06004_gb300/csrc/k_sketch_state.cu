@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(kBlock) k_query_at(const float* __restrict__ T
     for (int j = 0; j < r; ++j) {
       const uint64_t x = affine61(h.a[j], h.b[j], (uint32_t)i);
       const uint64_t y = affine61(h.a2[j], h.b2[j], (uint32_t)i);
-      v[j] = apply_sign(T[(size_t)j * c + bucket_of<false>(x, c, c - 1)], signbit_of(y));
+      v[j] = apply_sign(T[(size_t)j * c + (uint32_t)(x % c)], signbit_of(y));
     }
     for (int a = 1; a < r; ++a) {  // insertion sort
       const float tv = v[a];
@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(kBlock) k_add_sparse(float* __restrict__ T, co
     for (int j = 0; j < r; ++j) {
       const uint64_t x = affine61(h.a[j], h.b[j], (uint32_t)i);
       const uint64_t y = affine61(h.a2[j], h.b2[j], (uint32_t)i);
-      red_add_f32(T + (size_t)j * c + bucket_of<false>(x, c, c - 1), apply_sign(v, signbit_of(y)));
+      red_add_f32(T + (size_t)j * c + (uint32_t)(x % c), apply_sign(v, signbit_of(y)));
     }
   }
 }

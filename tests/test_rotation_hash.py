@@ -22,6 +22,19 @@ def _rot_mul(a8, i):
     return _rot_add((z & M32) << 32 | (w & M32), 8 * (z >> 32) + 8)
 
 
+def test_bucket_of_any_column_count():
+    """x mod c by the 64-bit inverse floor(2^64 / c): the quotient's estimate is at most 1 too small for
+    every x < 2^61, so the low words alone give the remainder."""
+    rng = np.random.default_rng(3)
+    cs = [3, 5, 6, 7, 777, 30_011, (1 << 26) - 1, (1 << 25) + 1] + [int(v) for v in rng.integers(3, 1 << 26, 50)]
+    for c in (c for c in cs if c & (c - 1)):
+        inv = M64 // c
+        xs = [0, 1, c - 1, c, c + 1, P61 - 1, P61 - 2, (P61 - 1) // c * c, (P61 - 1) // c * c - 1]
+        for x in xs + [int(v) % P61 for v in rng.integers(0, 1 << 62, 200)]:
+            r = ((x & M32) - ((x * inv >> 64) & M32) * c) & M32
+            assert (r - c if r >= c else r) == x % c
+
+
 def _rep(x):
     return 8 * (x + 1)
 
