@@ -203,12 +203,12 @@ gs_status insert_chains(const gs_sketch* sk, float* cells, int pitch, int W, int
   for (int j = j0; j < sk->r; ++j) {
     gs::ChainRow& row = p.row[j - j0];
     const gs::ChainShape ch = gs::choose_chain(sk->rotation[j], d, kMinStride, max_steps);
-    row.a = sk->h.a[j];
-    row.b = sk->h.b[j];
-    row.a2 = sk->h.a2[j];
-    row.b2 = sk->h.b2[j];
-    row.sa = gs::mulmod61(row.a, (uint64_t)ch.stride);
-    row.sa2 = gs::mulmod61(row.a2, (uint64_t)ch.stride);
+    row.a8 = 8 * sk->h.a[j];
+    row.b8 = 8 * sk->h.b[j];
+    row.a28 = 8 * sk->h.a2[j];
+    row.b28 = 8 * sk->h.b2[j];
+    row.sa8 = 8 * gs::mulmod61(sk->h.a[j], (uint64_t)ch.stride);
+    row.sa28 = 8 * gs::mulmod61(sk->h.a2[j], (uint64_t)ch.stride);
     row.cells = cells + (size_t)j * sk->c * pitch;
     row.stride = ch.stride;
     row.steps = ch.steps;

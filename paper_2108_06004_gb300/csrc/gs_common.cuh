@@ -43,6 +43,55 @@ __device__ __forceinline__ uint64_t step61(uint64_t x, uint64_t a) {
   return x >= kP61 ? x - kP61 : x;
 }
 
+// ---- the same by carries ------------------------------------------------------------------
+// For the kernels that are bound by their integer instructions (k_query_bits, k_insert_chain; k_query,
+// which is bound by its reads, took 4 % longer with it).  A hash value x in [0, p),
+// p = 2^61 - 1, is held as Y = 8 (x + 1), which lies in [8, 2^64 - 8].  For a residue s the 64-bit sum
+// Y + 8 s = 8 (x + s + 1) overflows exactly when x + s >= p, and then (x + s) mod p is represented by
+// the wrapped sum plus 8, since 8 p = 2^64 - 8.  So an addition and its carry-out reduce exactly,
+// without a compare, and the low word of Y alone gives the bucket and the sign.
+struct Rot {
+  uint32_t lo, hi;
+};
+
+// The representation of (x + s) mod p from that of x; s8 = 8 s, s in [0, p).
+__device__ __forceinline__ Rot rot_add(Rot y, uint64_t s8) {
+  uint32_t lo, hi, carry;
+  asm("add.cc.u32 %0, %3, %5;\n\taddc.cc.u32 %1, %4, %6;\n\taddc.u32 %2, 0, 0;"
+      : "=r"(lo), "=r"(hi), "=r"(carry)
+      : "r"(y.lo), "r"(y.hi), "r"((uint32_t)s8), "r"((uint32_t)(s8 >> 32)));
+  Rot out;
+  asm("add.cc.u32 %0, %2, %4;\n\taddc.u32 %1, %3, 0;" : "=r"(out.lo), "=r"(out.hi) : "r"(lo), "r"(hi), "r"(8u * carry));
+  return out;
+}
+
+// The low word of rot_add.
+__device__ __forceinline__ uint32_t rot_add_lo(Rot y, uint64_t s8) {
+  uint32_t lo, carry;
+  asm("{\n\t.reg .u32 hi;\n\tadd.cc.u32 %0, %2, %4;\n\taddc.cc.u32 hi, %3, %5;\n\taddc.u32 %1, 0, 0;\n\t}"
+      : "=r"(lo), "=r"(carry)
+      : "r"(y.lo), "r"(y.hi), "r"((uint32_t)s8), "r"((uint32_t)(s8 >> 32)));
+  return lo + 8u * carry;
+}
+
+// The representation of a i mod p, from a8 = 8 a, for i < 2^32: 8 a i = h 2^64 + l with h < 2^32, and
+// 2^64 is 8 modulo 2^64 - 8, so l + 8 h + 8 with its carry folded in as above (l / 8 + h < 2 p).
+__device__ __forceinline__ Rot rot_mul(uint64_t a8, uint32_t i) {
+  const uint64_t w = (uint64_t)(uint32_t)a8 * i;
+  const uint64_t z = (uint64_t)(uint32_t)(a8 >> 32) * i + (w >> 32);
+  return rot_add(Rot{(uint32_t)w, (uint32_t)z}, 8ull * (uint32_t)(z >> 32) + 8ull);
+}
+
+// The representation of (a i + b) mod p, and its low word.
+__device__ __forceinline__ Rot rot_at(uint64_t a8, uint64_t b8, uint32_t i) { return rot_add(rot_mul(a8, i), b8); }
+__device__ __forceinline__ uint32_t rot_at_lo(uint64_t a8, uint64_t b8, uint32_t i) {
+  return rot_add_lo(rot_mul(a8, i), b8);
+}
+
+// From the low word: the bucket for c a power of two, and the sign bit (bit 31 set when x is odd).
+__device__ __forceinline__ uint32_t rot_bucket(uint32_t lo, uint32_t cmask) { return ((lo >> 3) - 1u) & cmask; }
+__device__ __forceinline__ uint32_t rot_signbit(uint32_t lo) { return (~lo & 8u) << 28; }
+
 // x mod c.  For c not a power of two, with cinv = floor(2^64 / c): the estimate x * cinv >> 64 of the
 // quotient is at most 1 below it (x < 2^61), so the remainder needs one correction.
 template <bool POW2>
@@ -145,8 +194,8 @@ struct InsertParams {
 
 // Rows inserted by chains of coordinates (k_insert_chain), in launch order.
 struct ChainRow {
-  uint64_t a, b, a2, b2;  // the row's hash coefficients
-  uint64_t sa, sa2;       // a * stride and a2 * stride mod p: one step along a chain
+  uint64_t a8, b8, a28, b28;  // 8 times the row's hash coefficients
+  uint64_t sa8, sa28;         // 8 (a * stride mod p), 8 (a2 * stride mod p): one step along a chain
   float* cells;           // the row's cells, ChainParams::pitch floats apart
   int64_t stride;         // coordinates between two steps of a chain
   int32_t steps;          // coordinates of a chain

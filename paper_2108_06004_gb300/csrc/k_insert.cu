@@ -409,48 +409,49 @@ __global__ void __launch_bounds__(kChainBlock) k_insert_chain(const __grid_const
   const ChainRow& row = prm.row[ri];
   const uint32_t blk = blockIdx.x - row.first_block;
   const uint32_t seg = blk / row.tiles;  // segments of stride * steps coordinates
-  const int64_t S = row.stride;
-  const int64_t t = (int64_t)(blk - seg * row.tiles) * kChainBlock + threadIdx.x;
-  int64_t i = (int64_t)seg * row.steps * S + t;
-  if (t >= S || i >= prm.d) return;
+  const uint32_t S = (uint32_t)row.stride;
+  const uint32_t t = (blk - seg * row.tiles) * kChainBlock + threadIdx.x;
+  const int64_t start = (int64_t)seg * row.steps * row.stride + t;
+  if (t >= S || start >= prm.d) return;
+  uint32_t i = (uint32_t)start;
+  const uint32_t left = ((uint32_t)prm.d - 1u - i) / S;  // steps of this chain that the vector still holds
+  uint32_t n = left < (uint32_t)row.steps - 1u ? left : (uint32_t)row.steps - 1u;
   const size_t pitch = W == 1 ? (size_t)prm.pitch : (size_t)W;
   const uint64_t pol = prm.resident ? policy_normal() : policy_evict_first();
   const uint64_t pol_table = policy_evict_last();
-  uint64_t x = affine61(row.a, row.b, (uint32_t)i);
-  uint64_t y = affine61(row.a2, row.b2, (uint32_t)i);
-  uint32_t cur = (uint32_t)x & prm.cmask;
+  Rot x = rot_at(row.a8, row.b8, i), y = rot_at(row.a28, row.b28, i);
+  const auto cell = [&](uint32_t place) { return row.cells + (size_t)((place - 1u) & prm.cmask) * pitch; };
+  uint32_t cur = (x.lo >> 3) & prm.cmask;  // the place of the cell being summed: (bucket + 1) mod c
   float acc[W], v[W];
 #pragma unroll
   for (int w = 0; w < W; ++w) {
     acc[w] = 0.f;
     v[w] = w < prm.nw ? ld_hinted(prm.e[w] + i, pol) : 0.f;
   }
-  int n = row.steps;
   while (true) {
     float next[W];
-    i += S;
-    const bool more = --n > 0 && i < prm.d;
-    if (more) {
+    if (n > 0) {
+      i += S;
 #pragma unroll
       for (int w = 0; w < W; ++w) next[w] = w < prm.nw ? ld_hinted(prm.e[w] + i, pol) : 0.f;
     }
-    const uint32_t b = (uint32_t)x & prm.cmask;
-    if (b != cur) {
-      red_cell<W>(row.cells + (size_t)cur * pitch, acc, pol_table);
-      cur = b;
+    const uint32_t place = (x.lo >> 3) & prm.cmask;
+    if (place != cur) {
+      red_cell<W>(cell(cur), acc, pol_table);
+      cur = place;
 #pragma unroll
       for (int w = 0; w < W; ++w) acc[w] = 0.f;
     }
-    const float sg = __uint_as_float(0x3F800000u | signbit_of(y));
+    const float sg = __uint_as_float(0x3F800000u | rot_signbit(y.lo));
 #pragma unroll
     for (int w = 0; w < W; ++w) acc[w] = fmaf(v[w], sg, acc[w]);  // sg is +-1: rounds as an addition
-    if (!more) break;
-    x = step61(x, row.sa);
-    y = step61(y, row.sa2);
+    if (n-- == 0) break;
+    x = rot_add(x, row.sa8);
+    y = rot_add(y, row.sa28);
 #pragma unroll
     for (int w = 0; w < W; ++w) v[w] = next[w];
   }
-  red_cell<W>(row.cells + (size_t)cur * pitch, acc, pol_table);
+  red_cell<W>(cell(cur), acc, pol_table);
 }
 
 // Shared-memory-staged insert (the alternative to k_accumulate_insert_coop's direct cell
