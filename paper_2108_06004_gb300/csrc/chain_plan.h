@@ -12,6 +12,7 @@
 // Everything here only chooses strides; a poor choice costs time, never a result.
 #pragma once
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <vector>
@@ -31,24 +32,25 @@ inline std::vector<Convergent> rotation_convergents(uint64_t a, uint32_t c) {
   const u128 p = ((u128)1 << 61) - 1;
   const u128 den = p * c;
   const u128 num = ((u128)(a % c)) * p + a;  // < den
+  // q_n num is a multiple of den plus (-1)^n times the n-th remainder of the expansion
   std::vector<Convergent> out;
   u128 x = den, y = num;
   int64_t q0 = 0, q1 = 1;  // denominators of the last two convergents
-  const auto drift = [&](int64_t q) {
-    const u128 s = (u128)q * num % den;      // < 2^31 * 2^87
-    return s <= den / 2 ? (double)s / (double)p : -((double)(den - s) / (double)p);
-  };
-  out.push_back({1, drift(1)});
+  double sign = 1.0;
+  out.push_back({1, (double)y / (double)p});
   while (y != 0) {
     const u128 k = x / y;
     const u128 next = k * (u128)q1 + (u128)q0;
     if (next >= ((u128)1 << 31)) break;
-    const u128 t = x % y;
+    const u128 t = x - k * y;
     x = y;
     y = t;
     q0 = q1;
     q1 = (int64_t)next;
-    if (q1 > out.back().q) out.push_back({q1, drift(q1)});
+    sign = -sign;
+    const Convergent v = {q1, sign * ((double)y / (double)p)};
+    if (q1 > out.back().q) out.push_back(v);
+    else out.back() = v;
   }
   return out;
 }
@@ -86,6 +88,50 @@ inline ChainShape choose_chain(const std::vector<Convergent>& cv, int64_t d, int
     int64_t k1 = q0 >= min_stride ? 1 : (min_stride - q0 + q - 1) / q;
     if (k1 < 1) k1 = 1;
     if (k1 <= a) consider(k1 * q + q0, (double)k1 * cv[n].delta + cv[n - 1].delta);
+  }
+  return best;
+}
+
+// Strides with |drift| < 1/2 that are small combinations k q_n + l q_{n-1} of two neighbouring
+// convergents, ascending.
+inline std::vector<Convergent> slow_strides(const std::vector<Convergent>& cv, int64_t min_stride) {
+  std::vector<Convergent> out;
+  for (size_t n = 0; n < cv.size(); ++n)
+    for (int64_t k = 1; k <= 4; ++k)
+      for (int64_t l = 0; l <= (n > 0 ? 2 : 0); ++l) {
+        const int64_t q = k * cv[n].q + (l ? l * cv[n - 1].q : 0);
+        const double delta = (double)k * cv[n].delta + (l ? (double)l * cv[n - 1].delta : 0.0);
+        if (q >= min_stride && q < ((int64_t)1 << 31) && std::fabs(delta) < 0.5) out.push_back({q, delta});
+      }
+  std::sort(out.begin(), out.end(), [](const Convergent& x, const Convergent& y) { return x.q < y.q; });
+  return out;
+}
+
+// A walk that serves two rows: i = base + m * inner + n * outer with base < inner, base + m * inner < outer,
+// m < inner_steps and n < outer_steps, and the same again from every multiple of outer * outer_steps.
+// Along m the first row keeps its buckets, along n the second.
+struct PairShape {
+  int64_t inner = 0, outer = 0;
+  int32_t inner_steps = 0, outer_steps = 0;
+  double changes = 2.0;  // expected bucket changes per coordinate, both rows
+};
+
+inline PairShape choose_pair(const std::vector<Convergent>& first, const std::vector<Convergent>& second, int64_t d,
+                             int max_inner, int64_t max_steps) {
+  PairShape best;
+  for (const Convergent& o : second) {
+    if (o.q >= d) break;
+    for (const Convergent& s : first) {
+      if (s.q >= o.q) break;
+      const int64_t m = (o.q + s.q - 1) / s.q;
+      if (m > max_inner) continue;
+      int64_t n = (d + o.q - 1) / o.q;
+      if (n * m > max_steps) n = max_steps / m;
+      if (n < 1) continue;
+      const double reach = std::min((double)n, (double)d / (double)o.q);
+      const double changes = std::fabs(s.delta) + (double)s.q / (double)o.q + std::fabs(o.delta) + 1.0 / reach;
+      if (changes < best.changes) best = {s.q, o.q, (int32_t)m, (int32_t)n, changes};
+    }
   }
   return best;
 }

@@ -23,6 +23,7 @@ struct gs_sketch {
   // c a power of two: the convergents of every row's rotation (chain_plan.h) by one coordinate and
   // by a quad of four, else empty
   std::vector<std::vector<gs::Convergent>> rotation, quad_rotation;
+  std::vector<std::vector<gs::Convergent>> slow;  // slow_strides of every row
 };
 
 // Events recorded between the phases of a step while it is captured into a plan, where each
@@ -388,7 +389,7 @@ gs_status step_impl(gs_sketch* sk, float* const* m, float* const* e, const float
                                          sel.l2sq_out, ws, s, &marks.ev[kQueryBegin])) != cudaSuccess)
       return cuda_fail(err, "HEAVYMIX query launch");
   } else if ((err = gs::launch_query_topk(sk->merged, sk->h, sk->r, (uint32_t)sk->c, d, k, idx, est, ws, s,
-                                          &marks.ev[kQueryBegin])) != cudaSuccess) {
+                                          sk->slow, &marks.ev[kQueryBegin])) != cudaSuccess) {
     return cuda_fail(err, "query/top-k launch");
   }
   gs::GatherParams gp;
@@ -470,7 +471,7 @@ gs_status sketched_state_impl(gs_sketch* workers, gs_sketch* momentum, gs_sketch
     return cuda_fail(err, "sketch accumulate launch");
   // top-k of the estimate from E; delta = that estimate at the selected coordinates
   if ((err = gs::launch_query_topk(error->merged, error->h, error->r, (uint32_t)error->c, d, k, idx, nullptr,
-                                   ws, s, &marks.ev[kQueryBegin])) != cudaSuccess)
+                                   ws, s, error->slow, &marks.ev[kQueryBegin])) != cudaSuccess)
     return cuda_fail(err, "query/top-k launch");
   const float* est = static_cast<const float*>(ws);  // the query keeps est at the ws start
   if ((err = gs::launch_take(est, d, idx, k, vals, s)) != cudaSuccess) return cuda_fail(err, "take launch");
@@ -733,6 +734,7 @@ gs_status gs_sketch_create(int32_t r, int32_t c, uint64_t seed, int32_t workers,
   if (gs::is_pow2((uint32_t)c))
     for (int j = 0; j < r; ++j) {
       sk->rotation.push_back(gs::rotation_convergents(sk->h.a[j], (uint32_t)c));
+      sk->slow.push_back(gs::slow_strides(sk->rotation.back(), kMinStride));
       sk->quad_rotation.push_back(gs::rotation_convergents(gs::mulmod61(4, sk->h.a[j]), (uint32_t)c));
     }
   const int W = group_width ? group_width : choose_group_width(r, c, workers);
@@ -987,7 +989,7 @@ gs_status gs_query_topk(const gs_sketch* sk, int64_t d, int64_t k, int64_t* idx_
   if (workspace_bytes < gs::query_topk_workspace_bytes(d, k))
     return fail(GS_ERR_INVALID_ARG, "workspace too small: need " + std::to_string(gs::query_topk_workspace_bytes(d, k)));
   cudaError_t e = gs::launch_query_topk(sk->merged, sk->h, sk->r, (uint32_t)sk->c, d, k, idx_out, est_out, workspace,
-                                        as_stream(stream));
+                                        as_stream(stream), sk->slow);
   if (e != cudaSuccess) return cuda_fail(e, "query/top-k launch");
   return GS_OK;
   GS_GUARD_END
@@ -1037,7 +1039,7 @@ gs_status gs_query_topk_noalloc(const gs_sketch* sk, int64_t d, int64_t k, int64
   if (!est_out) return fail(GS_ERR_INVALID_ARG, "est_out is required by gs_query_topk_noalloc");
   GS_TRY(check_vec(est_out, "est_out"));
   cudaError_t e = gs::launch_query_topk_noalloc(sk->merged, sk->h, sk->r, (uint32_t)sk->c, d, k, idx_out, est_out,
-                                                as_stream(stream));
+                                                as_stream(stream), sk->slow);
   if (e != cudaSuccess) return cuda_fail(e, "query/top-k (no-allocation variant)");
   return GS_OK;
   GS_GUARD_END

@@ -9,6 +9,7 @@
 #include "gs_sketch.h"
 
 #include <utility>
+#include <vector>
 
 namespace gs {
 
@@ -221,6 +222,9 @@ struct ChainParams {
   ChainRow row[GS_MAX_ROWS];
 };
 
+struct Convergent;
+typedef std::vector<std::vector<Convergent>> RowStrides;  // per row, see slow_strides
+
 struct MergeParams {
   const float* tables;   // all groups, [group][r][c][W]
   float* merged;         // [r][c]
@@ -293,11 +297,13 @@ cudaError_t launch_query_at(const float* T, const HashCoeffs& h, int r, uint32_t
 cudaError_t launch_add_sparse(float* T, const HashCoeffs& h, int r, uint32_t c, const int64_t* idx, const float* vals,
                               int64_t k, float scale, cudaStream_t s);
 cudaError_t launch_take(const float* src, int64_t n, const int64_t* idx, int64_t k, float* out, cudaStream_t s);
+// slow: the slow strides of every row (empty unless c is a power of two).
 // marks (nullable): three events recorded, when set, before the query, between the query
 // (sample, median query, repair check) and the selection, and after the selection.
 cudaError_t launch_query_topk(const float* merged, const HashCoeffs& h, int r, uint32_t c,
                               int64_t d, int64_t k, int64_t* idx_out, float* est_out,
-                              void* workspace, cudaStream_t s, const cudaEvent_t* marks = nullptr);
+                              void* workspace, cudaStream_t s, const RowStrides& slow,
+                              const cudaEvent_t* marks = nullptr);
 // Request-ceiling probe of the median query: its loads (all r rows) without median, store or
 // histogram; out receives one float per CTA (out_floats must cover the grid).  c a power of two.
 cudaError_t launch_query_ceiling_probe(const float* merged, const HashCoeffs& h, int r, uint32_t c, int64_t d,
@@ -313,7 +319,7 @@ cudaError_t launch_query_heavymix(const float* merged, const HashCoeffs& h, int 
 // d <= GS_NOALLOC_MAX_DIM.  The first call on a device looks up the array's address.
 cudaError_t launch_query_topk_noalloc(const float* merged, const HashCoeffs& h, int r, uint32_t c,
                                       int64_t d, int64_t k, int64_t* idx_out, float* est_out,
-                                      cudaStream_t s);
+                                      cudaStream_t s, const RowStrides& slow);
 
 inline uint64_t bucket_inverse(uint32_t c) { return c > 1 ? ~0ull / c : 0; }  // floor(2^64 / c) unless c is a power of two
 inline bool is_pow2(uint32_t c) { return c && !(c & (c - 1)); }

@@ -409,6 +409,224 @@ __global__ void __launch_bounds__(kBlock, R <= 7 ? 4 : 1) k_query(const __grid_c
   if (prm.pick) last_block_pick(prm.hist, 11, prm.st, 0, prm.k);
 }
 
+// ---- the query along a walk that serves two rows ---------------------------------------------
+// Where the table is too large for k_query_bits, or every estimate is wanted, the query is bound by
+// its reads of table cells, one sector request from L1 to L2 each.  A walk along which two rows keep
+// their buckets (PairShape in chain_plan.h) needs a new cell of these rows for about a quarter of the
+// coordinates only: the inner row's cell stays in a register, the outer row's in shared memory, one
+// slot per inner step.  Each lane holds one coordinate; the hash values move by constant steps.
+// PRUNE: only the first kF rows are read here; the coordinates that they do not settle are queued
+// per warp with the cells read, and resolved 32 at a time, so that the later rows' work is done with
+// full warps.
+// Query in ms, k_query / here: all rows, d = 25,557,032, r = 5, c = 2^18 0.443 / 0.403; pruning, d =
+// 138,357,544, r = 7, c = 2^20 2.26 / 1.81, d = 83,311,104, r = 5, c = 2^21 1.01 / 0.83.  The walk's own
+// instructions now take about as long as the reads that are left; without the second coordinate in
+// flight the first of these took 0.423.
+constexpr int kWalkMaxRows = 9;
+constexpr int kWalkSlots = 8;  // inner steps at most
+
+struct WalkRow {
+  uint64_t a8, b8, a28, b28;   // 8 times the hash coefficients
+  uint64_t sa8, sa28;          // one inner step
+  uint64_t ja8[2], ja28[2];    // from the last inner step of a round to the next round: after inner_steps
+                               // steps, and after one fewer
+  const float* cells;
+};
+
+struct WalkParams {
+  uint32_t inner, outer;
+  int32_t inner_steps, outer_steps;
+  uint32_t tiles;              // CTAs across the inner stride
+  WalkRow row[kWalkMaxRows];   // the inner row, the outer row, the others
+};
+
+template <int R, bool PRUNE>
+__global__ void __launch_bounds__(kBlock, R <= 7 ? 3 : 2) k_query_walk(const __grid_constant__ QueryParams prm,
+                                                                      const __grid_constant__ WalkParams wk) {
+  grid_begin();
+  constexpr int kF = R / 2 + 1;
+  constexpr int NR = PRUNE ? kF : R;
+  constexpr int kEntry = kF + 1;
+  __shared__ uint32_t sh[kBins];
+  __shared__ float slot_cell[kWalkSlots][kBlock];
+  __shared__ uint32_t slot_place[kWalkSlots][kBlock];
+  __shared__ uint32_t queues[PRUNE ? kBlock / 32 : 1][PRUNE ? kEntry : 1][64];
+  for (int b = threadIdx.x; b < kBins; b += blockDim.x) sh[b] = 0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const uint32_t below = (1u << lane) - 1u;
+  const uint32_t d = (uint32_t)prm.d, S0 = wk.inner, S1 = wk.outer;
+  const uint32_t pk = PRUNE ? prune_key_of(prm) : 0u;
+  const uint32_t seg = blockIdx.x / wk.tiles;
+  const uint32_t base = (blockIdx.x - seg * wk.tiles) * kBlock + threadIdx.x;
+  const int64_t start = (int64_t)seg * wk.outer_steps * S1 + base;
+  const bool on = base < S0 && start < prm.d;
+  uint32_t i = on ? (uint32_t)start : 0u;
+  Rot x[NR], y[NR];
+#pragma unroll
+  for (int s = 0; s < NR; ++s) {
+    x[s] = rot_at(wk.row[s].a8, wk.row[s].b8, i);
+    y[s] = rot_at(wk.row[s].a28, wk.row[s].b28, i);
+  }
+  uint32_t (*queue)[64] = queues[PRUNE ? threadIdx.x >> 5 : 0];
+  uint32_t queued = 0;  // the same in every lane of the warp
+  uint32_t zeros = 0;   // this lane's markers: keys of bin 0
+  const auto drain = [&](uint32_t n) {
+    uint32_t bin = kNone;
+    if ((uint32_t)lane < n) {
+      const uint32_t at = queued + lane, c = queue[0][at];
+      float v[R];
+      int lt = 0, gt = 0, rows = kF;
+#pragma unroll
+      for (int j = 0; j < kF; ++j) {
+        v[j] = __uint_as_float(queue[1 + j][at]);
+        tally(v[j], pk, lt, gt);
+      }
+      bool done = pk != 0u && lt >= kF && gt >= kF;
+#pragma unroll
+      for (int j = kF; j < R; ++j) {
+        v[j] = 0.f;
+        if (!done) {
+          v[j] = signed_cell(prm, j, c);
+          tally(v[j], pk, lt, gt);
+          ++rows;
+        }
+        if (j + 1 < R) done = done || (pk != 0u && lt >= kF && gt >= kF);
+      }
+      const float m = done ? __uint_as_float(pruned_marker(rows, rows)) : median_of<R>(v);
+      prm.est[c] = m;
+      if (done) ++zeros;
+      else bin = key_of(m) >> kL1Shift;
+    }
+    hist_add(sh, bin);
+  };
+  float cell0 = 0.f;
+  uint32_t place0 = 0xFFFFFFFFu;
+  uint32_t round = i;  // the coordinate at m = 0
+  int m = 0, n = 0;
+  bool live = on;
+  // A coordinate whose cells are on their way.  Two are kept, so that the reads of one overlap the
+  // examination of the other; nothing here waits for a cell before the next one's reads are out.
+  struct Flight {
+    float raw[NR];
+    uint32_t i, m, signs;
+    bool held, moved, fresh;  // a coordinate at all; the inner row, the outer row in a new bucket
+  };
+  // reads the cells of the walk's coordinate, then moves the walk to the next one
+  const auto fetch = [&](Flight& f) {
+    f.held = live;
+    if (!live) return;
+    f.i = i;
+    f.m = (uint32_t)m;
+#pragma unroll
+    for (int s = 2; s < NR; ++s) f.raw[s] = __ldg(wk.row[s].cells + rot_bucket(x[s].lo, prm.cmask));
+    const uint32_t p0 = (x[0].lo >> 3) & prm.cmask, p1 = (x[1].lo >> 3) & prm.cmask;
+    f.moved = p0 != place0;
+    if (f.moved) {
+      place0 = p0;
+      f.raw[0] = __ldg(wk.row[0].cells + ((p0 - 1u) & prm.cmask));
+    }
+    f.fresh = n == 0 || slot_place[m][threadIdx.x] != p1;
+    if (f.fresh) {
+      f.raw[1] = __ldg(wk.row[1].cells + ((p1 - 1u) & prm.cmask));
+      slot_place[m][threadIdx.x] = p1;
+    }
+    f.signs = 0;
+#pragma unroll
+    for (int s = 0; s < NR; ++s) f.signs |= (rot_signbit(y[s].lo) >> 31) << s;
+    // the next inner step, or the next round; m * S0 + base = i - round + base
+    const bool inside = i - round + base + S0 < S1 && i + S0 < d;
+    const bool full = m == wk.inner_steps - 1;
+    if (inside) {
+      i += S0;
+      ++m;
+    } else {
+      // where the vector ends before the round does, the next round lies beyond it as well
+      i = round + S1;
+      round = i;
+      m = 0;
+      ++n;
+      live = n < wk.outer_steps && i < d;
+    }
+#pragma unroll
+    for (int s = 0; s < NR; ++s) {
+      const WalkRow& r = wk.row[s];
+      x[s] = rot_add(x[s], inside ? r.sa8 : full ? r.ja8[0] : r.ja8[1]);
+      y[s] = rot_add(y[s], inside ? r.sa28 : full ? r.ja28[0] : r.ja28[1]);
+    }
+  };
+  const auto examine = [&](Flight& f) {
+    bool open = false;
+    uint32_t bin = kNone;
+    float v[R];
+#pragma unroll
+    for (int s = 0; s < NR; ++s) v[s] = 0.f;
+    if (f.held) {
+      if (f.moved) cell0 = f.raw[0];
+      v[0] = cell0;
+      if (f.fresh) slot_cell[f.m][threadIdx.x] = f.raw[1];  // a slot serves again one round later
+      else f.raw[1] = slot_cell[f.m][threadIdx.x];
+#pragma unroll
+      for (int s = 1; s < NR; ++s) v[s] = f.raw[s];
+#pragma unroll
+      for (int s = 0; s < NR; ++s) v[s] = apply_sign(v[s], (f.signs >> s) << 31);
+      if (PRUNE) {
+        int lt = 0, gt = 0;
+#pragma unroll
+        for (int s = 0; s < NR; ++s) tally(v[s], pk, lt, gt);
+        open = pk == 0u || lt < kF || gt < kF;
+        if (!open) {
+          prm.est[f.i] = __uint_as_float(pruned_marker(kF, kF));
+          ++zeros;
+        }
+      } else {
+        float t[R];
+#pragma unroll
+        for (int s = 0; s < R; ++s) t[s] = v[s];
+        const float e = median_of<R>(t);
+        prm.est[f.i] = e;
+        bin = key_of(e) >> kL1Shift;
+      }
+    }
+    if (PRUNE) {
+      const uint32_t who = __ballot_sync(kFull, open);
+      if (open) {
+        const uint32_t at = queued + __popc(who & below);
+        queue[0][at] = f.i;
+#pragma unroll
+        for (int j = 0; j < kF; ++j) queue[1 + j][at] = __float_as_uint(v[j]);
+      }
+      queued += __popc(who);
+      __syncwarp();
+      if (queued >= 32) {
+        queued -= 32;
+        drain(32);
+        __syncwarp();
+      }
+    } else {
+      hist_add(sh, bin);
+    }
+  };
+  Flight f0, f1;
+  fetch(f0);
+  while (__any_sync(kFull, f0.held)) {
+    fetch(f1);
+    examine(f0);
+    fetch(f0);
+    examine(f1);
+  }
+  if (PRUNE) {
+    const uint32_t n_left = queued;
+    queued = 0;
+    if (n_left) drain(n_left);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) zeros += __shfl_down_sync(kFull, zeros, o);
+    if (lane == 0 && zeros) atomicAdd(&sh[0], zeros);
+  }
+  hist_flush(sh, prm.hist, kBins);
+  if (prm.pick) last_block_pick(prm.hist, 11, prm.st, 0, prm.k);
+}
+
 // ---- the pruning query with the first rows classified in shared memory ---------------------
 // The settle rule needs, for each of the first f = r/2 + 1 cells of a coordinate, only which side
 // of the prune key t its value lies on: whether it counts below t, above -t, or both (|T| < t: the
@@ -1679,7 +1897,80 @@ constexpr ProbeLauncher ProbeTable<Rs...>::table[sizeof...(Rs)];
 constexpr int64_t kPruneMinDim = int64_t(1) << 22;
 bool can_prune(int r, uint32_t c, int64_t d) { return is_pow2(c) && r >= 3 && r <= GS_MAX_ROWS && d >= kPruneMinDim; }
 
-cudaError_t launch_query(const QueryParams& p, cudaStream_t s) {
+template <int R>
+cudaError_t launch_walk_r(const QueryParams& p, WalkParams& wk, cudaStream_t s) {
+  const int64_t span = (int64_t)wk.outer * wk.outer_steps;
+  wk.tiles = (wk.inner + kBlock - 1) / kBlock;
+  const uint32_t blocks = wk.tiles * (uint32_t)((p.d + span - 1) / span);
+  if (p.prune) launch(k_query_walk<R, true>, blocks, kBlock, s, p, wk);
+  else launch(k_query_walk<R, false>, blocks, kBlock, s, p, wk);
+  return cudaGetLastError();
+}
+
+typedef cudaError_t (*WalkLauncher)(const QueryParams&, WalkParams&, cudaStream_t);
+
+template <int... Rs>
+struct WalkTable {
+  static constexpr WalkLauncher table[sizeof...(Rs)] = {&launch_walk_r<Rs>...};
+};
+template <int... Rs>
+constexpr WalkLauncher WalkTable<Rs...>::table[sizeof...(Rs)];
+
+// The walk pays where the reads it saves outweigh its steps.  Query with its selection in us, k_query /
+// walk: all rows, r = 3, d = 4.2M, c = 2^16 79 / 85; r = 5, d = 2.1M, c = 2^16 72 / 73, d = 4.2M, c = 2^15
+// 105 / 106, c = 2^17 113 / 104, d = 25.6M, c = 2^20 494 / 463; r = 9, d = 4.2M 177 / 165.  Pruning reads
+// r/2 + 1 rows, so that two of them weigh more: r = 5, d = 25.6M, c = 2^20 395 / 342, r = 7, c = 2^18 510 / 444.
+constexpr int64_t kWalkQueryMinDim = int64_t(1) << 22;
+constexpr uint32_t kWalkQueryMinCols = 1u << 16;
+
+// The walk of a query, or false where k_query serves it.
+bool plan_walk(const QueryParams& p, const RowStrides& slow, WalkParams& wk) {
+  if (slow.empty() || p.keys || p.r < (p.prune ? 3 : 5) || p.r > kWalkMaxRows || p.d < kWalkQueryMinDim || p.c < kWalkQueryMinCols)
+    return false;
+  const int nr = p.prune ? p.r / 2 + 1 : p.r;
+  const int64_t max_steps = p.d / ((int64_t)device_info().sms * 1024 * 2);
+  PairShape best;
+  int first = 0, second = 1;
+  for (int f = 0; f < 2; ++f) {  // either of the first two rows as the inner one
+    const PairShape s = choose_pair(slow[f], slow[1 - f], p.d, kWalkSlots, max_steps < 64 ? max_steps : 64);
+    if (s.changes < best.changes) {
+      best = s;
+      first = f;
+      second = 1 - f;
+    }
+  }
+  if (best.changes > 1.0) return false;
+  std::memset(&wk, 0, sizeof(wk));
+  wk.inner = (uint32_t)best.inner;
+  wk.outer = (uint32_t)best.outer;
+  wk.inner_steps = best.inner_steps;
+  wk.outer_steps = best.outer_steps;
+  for (int s = 0; s < nr; ++s) {
+    const int j = s == 0 ? first : s == 1 ? second : s;
+    WalkRow& r = wk.row[s];
+    r.a8 = p.h8.a[j];
+    r.b8 = p.h8.b[j];
+    r.a28 = p.h8.a2[j];
+    r.b28 = p.h8.b2[j];
+    r.sa8 = 8 * mulmod61(p.h.a[j], (uint64_t)best.inner);
+    r.sa28 = 8 * mulmod61(p.h.a2[j], (uint64_t)best.inner);
+    for (int t = 0; t < 2; ++t) {
+      // inner_steps - 1 inner strides are less than the outer one, and inner_steps >= 2
+      const uint64_t jump = (uint64_t)(best.outer - (best.inner_steps - 1 - t) * best.inner);
+      r.ja8[t] = 8 * mulmod61(p.h.a[j], jump);
+      r.ja28[t] = 8 * mulmod61(p.h.a2[j], jump);
+    }
+    r.cells = p.T + (size_t)j * p.c;
+  }
+  return true;
+}
+
+cudaError_t launch_query(const QueryParams& p, const RowStrides& slow, cudaStream_t s) {
+  WalkParams wk;
+  if (plan_walk(p, slow, wk)) {
+    using T = WalkTable<3, 4, 5, 6, 7, 8, 9>;
+    return T::table[p.r - 3](p, wk, s);
+  }
   using T = QueryTable<1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16>;
   return T::table[p.r - 1](p, s);
 }
@@ -1829,7 +2120,7 @@ cudaError_t select_from_keys(const Workspace& w, const float* src, int vec, uint
 
 cudaError_t launch_query_topk(const float* merged, const HashCoeffs& h, int r, uint32_t c,
                               int64_t d, int64_t k, int64_t* idx_out, float* est_out,
-                              void* workspace, cudaStream_t s, const cudaEvent_t* marks) {
+                              void* workspace, cudaStream_t s, const RowStrides& slow, const cudaEvent_t* marks) {
   Workspace w = carve(workspace, d);
   float* est = est_out ? est_out : w.est;
   cudaError_t err = clear_selection(w, d, s);
@@ -1847,7 +2138,7 @@ cudaError_t launch_query_topk(const float* merged, const HashCoeffs& h, int r, u
   }
   if (qp.prune && query_uses_bits(r, c)) {
     if ((err = launch_query_bits(qp, w, s)) != cudaSuccess) return err;
-  } else if ((err = launch_query(qp, s)) != cudaSuccess) {
+  } else if ((err = launch_query(qp, slow, s)) != cudaSuccess) {
     return err;
   }
   if (qp.prune) {
@@ -1900,7 +2191,7 @@ cudaError_t launch_query_heavymix(const float* merged, const HashCoeffs& h, int 
   qp.theta = theta;
   qp.fill_seed = fill_seed;
   if (prune && query_uses_bits(r, c)) err = launch_query_bits(qp, w, s);
-  else err = launch_query(qp, s);
+  else err = launch_query(qp, RowStrides(), s);
   if (err != cudaSuccess) return err;
   if ((err = mark(marks, 1, s)) != cudaSuccess) return err;
   const float* src = reinterpret_cast<const float*>(keys);
@@ -1990,7 +2281,7 @@ cudaError_t noalloc_scratch(void** out) {
 
 cudaError_t launch_query_topk_noalloc(const float* merged, const HashCoeffs& h, int r, uint32_t c,
                                       int64_t d, int64_t k, int64_t* idx_out, float* est_out,
-                                      cudaStream_t s) {
+                                      cudaStream_t s, const RowStrides& slow) {
   if (d > GS_NOALLOC_MAX_DIM || est_out == nullptr) return cudaErrorInvalidValue;
   void* base = nullptr;
   cudaError_t err = noalloc_scratch(&base);
@@ -2009,7 +2300,7 @@ cudaError_t launch_query_topk_noalloc(const float* merged, const HashCoeffs& h, 
 
   QueryParams qp = make_query_params(merged, h, r, c, d, k, est_out, hist, st);
   qp.pick = selects_small(d) ? 0 : 1;
-  if ((err = launch_query(qp, s)) != cudaSuccess) return err;
+  if ((err = launch_query(qp, slow, s)) != cudaSuccess) return err;
   if (selects_small(d)) return select_small(est_out, qp.vec, 0x7FFFFFFFu, hist, st, 0, d, k, idx_out, s);
   const int hgrid = persistent_grid(k_hist, (d + 3) / 4 / kU, kBlock);
   launch(k_hist, hgrid, kBlock, s, est_out, d, qp.vec, st, hist + kBins, kL2Shift, 11, 1);
