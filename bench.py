@@ -53,6 +53,18 @@ def query_classifies(r: int, c: int) -> bool:
     (one more kernel, which writes the cell classes)."""
     return 3 <= r <= 16 and c >= 64 and (c & (c - 1)) == 0 and (r // 2 + 1) * c // 4 <= CLASS_BYTES
 
+
+
+def insert_rows(W: int, r: int, c: int, d: int) -> int:
+    """How many of the r rows (c a power of two) the accumulate pass of a group of W workers inserts;
+    the others go along chains of coordinates, which read the error vectors once more per row."""
+    if d * r <= 1 << 20:
+        return r
+    if d < 1 << 22:
+        return r if W == 16 else 0
+    return min(r if W == 16 else max(1, W // 2), (48 << 20) // (c * W * 4), r)
+
+
 VARIANTS = {
     "error_feedback": "S1-S6: per-worker momentum and error vectors, exact second round",
     "train": "S1-S7: as error_feedback, with the weight update fused into the second round",
@@ -285,9 +297,11 @@ class Runner:
         gs = self.gs
         self.sk = gs.gs_sketch_create(r, c, 20210813, P, group_width)
         info = gs.gs_sketch_info(self.sk)
-        self.W, self.rpp = info["group_width"], info["rows_per_pass"]
+        self.W = info["group_width"]
         self.groups = (P + self.W - 1) // self.W
-        self.passes = -(-r // self.rpp)
+        self.main_rows = None if variant == "sketched_state" else insert_rows(self.W, r, w.c, w.d)
+        # launches of a group's insert: the accumulate pass, and one more for the rows it leaves out
+        self.insert_launches = 1 if self.main_rows is None or self.main_rows == r else 2
         ws_bytes = gs.gs_step_workspace_size(d, k)
         if variant == "heavymix":
             ws_bytes = max(ws_bytes, gs.gs_query_heavymix_workspace_size(d, k))
@@ -426,16 +440,19 @@ class Runner:
 
 
 def launches_per_step(run: Runner, variant: str) -> int:
-    """Kernels of the library launched per step: insert (one per group and row pass, and per
-    worker batch), merge, the query and selection, the gather (sketched state: its own)."""
+    """Kernels of the library launched per step: insert (per group the accumulate pass and, for the
+    rows it leaves out, the chained insert), merge, the query and selection, the gather (sketched
+    state: its own)."""
     w = run.w
     prunes = variant != "heavymix" and w.d >= PRUNE_MIN_DIM and w.r >= 3 and (w.c & (w.c - 1)) == 0
-    inserts = run.groups * run.passes
+    inserts = run.groups * run.insert_launches
+    bits = w.d >= PRUNE_MIN_DIM and query_classifies(w.r, w.c)
+    select = 1 if w.d <= 3 << 19 else 6               # one cluster up to 1.5 * 2^20 coordinates
     if variant == "heavymix":
-        query = 3 + 6                                 # sumsq, theta, query (with the keys) + selection
+        query = 3 + int(bits) + select                # sumsq, theta, query (with the keys) + selection
     else:
         # query + selection (+ sample and repair check, + the cell classes)
-        query = 1 + 6 + (2 + int(query_classifies(w.r, w.c)) if prunes else 0)
+        query = 1 + select + (2 + int(bits) if prunes else 0)
     tail = 6 if variant == "sketched_state" else 1
     return inserts + 1 + query + tail
 
@@ -492,18 +509,19 @@ def rooflines(run: Runner, variant: str, ph: dict, peaks, peak_kind, probes: dic
     w = run.w
     P, d, r = w.P, w.d, w.r
     per_wc = 4.0 if variant == "sketched_state" else 20.0
-    moved_wc = per_wc + 4.0 * (run.passes - 1)   # every pass after the first re-reads e (or g)
+    # every chained row reads e (sketched state: g) once more
+    moved_wc = 4.0 * r if run.main_rows is None else per_wc + 4.0 * (r - run.main_rows)
     phase_s = ph["insert"] / 1e3
     phase_bytes = per_wc * P * d
     k1_gbs = phase_bytes / phase_s / 1e9
     cells = d * r * run.groups
-    nl = run.groups * run.passes
+    nl = run.groups * run.insert_launches
     k1 = {
         "kernel": ("k_accumulate + k_insert_staged (S1, then S2 staged in shared memory" if run.staged else
-                   "k_accumulate_insert_coop (insert only" if variant == "sketched_state" else
-                   "k_accumulate_insert_coop (fused S1+S2") + f", W={run.W}), the insert phase of a step: "
-                  f"{run.groups} group(s) x {run.passes} row pass(es)",
-        "row_passes": run.passes, "groups": run.groups, "launches_per_phase": nl,
+                   "k_insert_chain (insert only" if variant == "sketched_state" else
+                   "k_accumulate_chain / k_accumulate_insert_coop (fused S1+S2), k_insert_chain (the other rows")
+                  + f", W={run.W}), the insert phase of a step: {run.groups} group(s)",
+        "rows_in_accumulate_pass": run.main_rows, "groups": run.groups, "launches_per_phase": nl,
         "algorithmic_bytes_per_worker_coord": per_wc, "moved_bytes_per_worker_coord": moved_wc,
         "bound": "hbm", "achieved": round(k1_gbs, 1), "peak": peaks["hbm_gbs"], "unit": "GB/s",
         "frac": round(k1_gbs / peaks["hbm_gbs"], 4), "peak_source": peak_kind,
@@ -520,8 +538,9 @@ def rooflines(run: Runner, variant: str, ph: dict, peaks, peak_kind, probes: dic
     # the probe stands for the fused accumulate + insert; the sketched state inserts raw gradients
     ceil_ms = probes.get("insert_ms") if variant != "sketched_state" else None
     k1["co_bound"] = {
-        "kind": "SM->L2 requests: one cell reduction per (coordinate, row, group) plus the u, e stores and the loads",
-        "probe": "gs_insert_request_ceiling: the same kernels, grids, buckets and reductions with every vector access "
+        "kind": "SM->L2 requests of an insert by one reduction per (coordinate, row, group), with the u, e stores and "
+                "the loads; chained rows send about a tenth of the reductions, so the phase may be faster",
+        "probe": "gs_insert_request_ceiling: the kernels that insert every row so, with every vector access "
                  "folded into an L2-resident window (no HBM traffic)",
         "cell_updates_per_phase": cells,
         "achieved_G_cells_per_s": round(cells / phase_s / 1e9, 1),
@@ -545,7 +564,7 @@ def rooflines(run: Runner, variant: str, ph: dict, peaks, peak_kind, probes: dic
         ach = requests / (q_ms / 1e3) / 1e9
         q = {
             "kernel": ((f"k_qsample + k_pbits + k_query_bits<{r}> + k_repair (median query, S4)"
-                        if query_classifies(r, w.c) else f"k_qsample + k_query<{r}> + k_repair (median query, S4)")
+                        if query_classifies(r, w.c) else f"k_qsample + k_query_walk<{r}> + k_repair (median query, S4)")
                        if prunes else f"k_query<{r}> (S4)") +
                       (" and the S5 selection: eager, timed around the gs_query_topk call" if with_selection else ""),
             "bound": ("integer ALU pipe: the Mersenne hash of every row examined (the first rows' cells are "
@@ -676,7 +695,7 @@ def short_summary(res: dict, w) -> dict:
         "d": w.d, "P": w.P, "r": w.r, "c": w.c, "k": w.k, "steps": res["steps"], "launch": res["launch"],
         "value": res["value"], "unit": UNIT, "ms_per_step": res["ms_per_step"], "l2": res["l2"],
         "insert": {"avg_phase_ms": k1["avg_phase_ms"], "achieved": k1["achieved"], "frac": k1["frac"],
-                   "row_passes": k1["row_passes"], "groups": k1["groups"],
+                   "rows_in_accumulate_pass": k1["rows_in_accumulate_pass"], "groups": k1["groups"],
                    "moved_bytes_per_worker_coord": k1["moved_bytes_per_worker_coord"],
                    "request_ceiling_ms": k1["co_bound"]["peak_ms"], "frac_of_request_ceiling": k1["co_bound"]["frac"],
                    "request_ceiling_frac_of_hbm": k1["co_bound"]["peak_frac_of_hbm"]},

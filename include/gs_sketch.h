@@ -70,8 +70,8 @@ typedef struct gs_plan gs_plan;     /* opaque: one step captured into a CUDA gra
  * cell are adjacent and are updated by 16-byte vector reductions (G = group_width/4 lanes
  * together write a whole cell in one instruction); group_width 0 lets the library choose
  * (up to 16, no wider than the worker count rounded up to a power of two; 16 only when the
- * whole group table fits 48 MiB of L2, and halved while one table row exceeds 64 MiB).  The
- * fused insert updates as many rows per pass as fit 48 MiB, and at least one.
+ * whole group table fits 48 MiB of L2, and halved while one table row exceeds 64 MiB).
+ * rows_per_pass (gs_sketch_info) is the number of table rows that fit 48 MiB, and at least one.
  * On success *out owns device memory released by gs_sketch_destroy.
  * Errors: GS_ERR_INVALID_ARG (sizes, group_width not in {0,1,2,4,8,16}, out NULL),
  *         GS_ERR_OOM (allocation failed), GS_ERR_CUDA.  Synchronous. */
@@ -81,8 +81,9 @@ gs_status gs_sketch_create(int32_t r, int32_t c, uint64_t seed, int32_t workers,
 /* Release a sketch and its device memory.  NULL is accepted.  Synchronous. */
 gs_status gs_sketch_destroy(gs_sketch* sketch);
 
-/* Shape query: any output pointer may be NULL.  rows_per_pass is the number of rows the
- * fused insert updates per pass over the vectors. */
+/* Shape query: any output pointer may be NULL.  rows_per_pass is the number of rows the fused
+ * insert updates per pass over the vectors when it sends one reduction per coordinate and row (c
+ * not a power of two, or gradients read from host memory). */
 gs_status gs_sketch_info(const gs_sketch* sketch, int32_t* r, int32_t* c, int32_t* workers,
                          int32_t* group_width, int32_t* rows_per_pass);
 
@@ -116,9 +117,10 @@ gs_status gs_sketch_insert(gs_sketch* sketch, int32_t worker, const float* vec, 
  * pointer arrays are HOST arrays of n_workers DEVICE pointers.  first_worker must be a
  * multiple of the group width, and the range must end on a group boundary or at the
  * last worker.  Per worker the result equals gs_accumulate followed by gs_sketch_insert
- * (up to the order of the fp32 atomic additions in the cells).  When the table is inserted
- * in several row passes, the first pass also accumulates and the later ones re-read the
- * updated error vectors. */
+ * (up to the order of the fp32 additions in the cells).  For c a power of two some or all rows
+ * are inserted along chains of coordinates that share a bucket, summed in registers before they
+ * reach the cell; these rows, and the rows of later passes over a table that is inserted in
+ * several, re-read the updated error vectors. */
 gs_status gs_accumulate_insert(gs_sketch* sketch, int32_t first_worker, int32_t n_workers,
                                float* const* momentum, float* const* error,
                                const float* const* grad, int64_t d, float rho,
@@ -416,15 +418,14 @@ gs_status gs_plan_query_times(gs_plan* plan, float* query_ms_out, float* select_
 gs_status gs_plan_destroy(gs_plan* plan);
 
 /* ---- measurement aid --------------------------------------------------------------- */
-/* The fused insert (gs_accumulate_insert over every group and row pass) is bound by the
- * requests its SMs send to L2: one cell reduction per (coordinate, row, group) and the
- * momentum and error stores, rather than by HBM bandwidth.  gs_insert_request_ceiling
- * measures the time of that request mix with HBM taken out: it runs the insert kernels of one
- * whole insert phase for d coordinates and all of the sketch's workers, with the same grids,
- * instructions, hash buckets and cell reductions, but with every vector access folded into an
+/* An insert that sends one cell reduction per (coordinate, row, group) beside the momentum and
+ * error stores is bound by the requests its SMs send to L2 rather than by HBM bandwidth.
+ * gs_insert_request_ceiling measures the time of that request mix with HBM taken out: it runs the
+ * kernels of such an insert phase (every row by reductions, in passes of rows_per_pass rows) for d
+ * coordinates and all of the sketch's workers, with every vector access folded into an
  * L2-resident window (GS_CEILING_WINDOW_FLOATS floats per vector).  Not a step of the method
- * (the paper has no counterpart); it only gives the insert's roofline a measured second
- * bound.  window: a device buffer of gs_insert_request_ceiling_window_size bytes, 256-byte
+ * (the paper has no counterpart): it is what the chained insert is compared with, and the bound
+ * of the rows that still go by reductions.  window: a device buffer of gs_insert_request_ceiling_window_size bytes, 256-byte
  * aligned, overwritten.  The worker tables are left unspecified: zero them before the next
  * insert.  *ms_out (host) receives the elapsed time of the phase, measured with events on
  * `stream`; the call synchronizes with them.  GS_ERR_INVALID_ARG unless the group width is

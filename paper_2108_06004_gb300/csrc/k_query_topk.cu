@@ -16,7 +16,10 @@
 //                 on the k-th largest |est| of this query, rounded down to a bin edge
 //   k_query       est_i for every i (fp32) + level-1 histogram + pick; when the estimate stays
 //                 in the workspace, a coordinate whose rows read so far bound its |est| below
-//                 the prune key skips its other rows and stores a marker (see below)
+//                 the prune key skips its other rows and stores a marker (see below).  In its place:
+//                 k_query_bits (pruning, the first rows' cells classified in shared memory),
+//                 k_query_walk (long vectors, along a walk that keeps two rows' cells) and
+//                 k_query_mod (c not a power of two)
 //   k_repair      runs only if the level-1 pick fell below the prune key: recomputes every
 //                 marked estimate in full, rebuilds the level-1 histogram and picks again
 //   k_cand        one pass over est: keys above the picked level-1 bin are selected for
@@ -27,6 +30,7 @@
 //   k_bm_count    per block of 65536 coordinates: bits set in each bitmap
 //   k_scan        one CTA: exclusive prefix sums over the blocks
 //   k_bm_write    every block writes its selected indices at their final positions
+// Up to d = 1.5 * 2^20 one launch of k_select_small replaces k_cand .. k_bm_write.
 // With the fixed scratch (gs_query_topk_noalloc), which cannot hold candidate lists, the
 // levels 2 and 3 and the final selection read est in full passes (k_hist, k_count, k_write).
 #include <cmath>

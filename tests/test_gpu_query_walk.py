@@ -1,7 +1,8 @@
 """The query along a walk that serves two rows, against the per-index query (gs_sketch_query_at), which
 shares none of its path: every estimate bit-equal, for each number of rows the walk serves (3 and 4 only
-where it prunes), ragged d, the smallest and a large number of columns; the pruning form (its estimate internal) selects the same
-coordinates, with every unpruned estimate equal and every marker below the k-th largest."""
+where it prunes), ragged d, the smallest and a large number of columns; the pruning form (its estimate
+internal) selects the same coordinates, with every unpruned estimate equal and every marker below the
+k-th largest."""
 
 import numpy as np
 import pytest
