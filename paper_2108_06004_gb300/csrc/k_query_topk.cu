@@ -693,10 +693,11 @@ __global__ void __launch_bounds__(kBlock) k_pbits(const float* __restrict__ T, u
 }
 
 // A coordinate i from its signs: its first kF cells by their bits, the later rows from the table
-// while it is undecided, and its full median when it does not settle.  Returns the estimate or
-// marker.
+// while it is undecided, and its full median when it does not settle.  Returns the marker (settled)
+// or the estimate: the value alone does not tell them apart, an estimate may have a marker's bits.
 template <int R>
-__device__ __forceinline__ float resolve(const QueryParams& prm, const uint32_t* sbits, uint32_t i, uint32_t pk) {
+__device__ __forceinline__ float resolve(const QueryParams& prm, const uint32_t* sbits, uint32_t i, uint32_t pk,
+                                         bool& settled) {
   constexpr int kF = R / 2 + 1;
   const uint32_t per_row = prm.c / 32;
   uint32_t cell[kF];  // bucket of each of the first kF rows, sign bit of the cell in bit 31
@@ -723,6 +724,7 @@ __device__ __forceinline__ float resolve(const QueryParams& prm, const uint32_t*
     }
     if (j + 1 < R) done = done || (pk != 0u && lt >= kF && gt >= kF);
   }
+  settled = done;
   if (done) return __uint_as_float(pruned_marker(rows, rows - kF));
 #pragma unroll
   for (int j = 0; j < kF; ++j)
@@ -765,10 +767,9 @@ __global__ void __launch_bounds__(kBitsBlock, 1) k_query_bits(const __grid_const
     n3 += __popc(m);
     if (who) queue[kQueue - n3 + __popc(m & below)] = i;
   };
-  // the estimate or marker m of coordinate i, and its key in HEAVYMIX
-  const auto record = [&](uint32_t i, float m) {
+  // the estimate of coordinate i or its marker, and its key in HEAVYMIX
+  const auto record = [&](uint32_t i, float m, bool marker) {
     prm.est[i] = m;
-    const bool marker = is_pruned(__float_as_uint(m));
     if (HM) {
       const uint32_t key = heavy_key(marker ? 0.f : m, theta, prm.fill_seed, (uint64_t)i);
       prm.keys[i] = key;
@@ -781,7 +782,9 @@ __global__ void __launch_bounds__(kBitsBlock, 1) k_query_bits(const __grid_const
     uint32_t bin = kNone;
     if (active) {
       const uint32_t i = queue[kQueue - n3 + lane];
-      bin = record(i, resolve<R>(prm, sbits, i, pk));
+      bool done;
+      const float m = resolve<R>(prm, sbits, i, pk, done);
+      bin = record(i, m, done);
     }
     hist_add(sh, bin);
   };
@@ -793,7 +796,7 @@ __global__ void __launch_bounds__(kBitsBlock, 1) k_query_bits(const __grid_const
       const uint32_t x = rot_at_lo(prm.h8.a[kF], prm.h8.b[kF], i);
       open = key_of(__ldg(prm.T + (size_t)kF * prm.c + rot_bucket(x, prm.cmask))) >= pk;
       if (!open) {
-        const uint32_t bin = record(i, __uint_as_float(pruned_marker(kF + 1, 1)));
+        const uint32_t bin = record(i, __uint_as_float(pruned_marker(kF + 1, 1)), true);
         if (HM) atomicAdd(&sh[bin], 1u);
       }
     }
