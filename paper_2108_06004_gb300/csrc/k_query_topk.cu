@@ -30,12 +30,14 @@
 //   k_bm_count    per block of 65536 coordinates: bits set in each bitmap
 //   k_scan        one CTA: exclusive prefix sums over the blocks
 //   k_bm_write    every block writes its selected indices at their final positions
-// Up to d = 1.5 * 2^20 one launch of k_select_small replaces k_cand .. k_bm_write.
+// Up to d = 1.5 * 2^20 one launch of k_select_small replaces k_cand .. k_bm_write, where the device can
+// hold its cluster.
 // With the fixed scratch (gs_query_topk_noalloc), which cannot hold candidate lists, the
 // levels 2 and 3 and the final selection read est in full passes (k_hist, k_count, k_write).
 #include <cmath>
 #include <cstring>
 #include <mutex>
+#include <unordered_map>
 
 #include <cooperative_groups.h>
 #include <cuda.h>
@@ -1338,8 +1340,6 @@ constexpr int kSmallThreads = 1024;
 constexpr int kSmallList = 16384;                   // candidates kept per CTA
 constexpr int64_t kSmallMaxDim = int64_t(3) << 19;  // 3072 bitmap words per CTA
 
-bool selects_small(int64_t d) { return d <= kSmallMaxDim; }
-
 struct SmallShared {
   uint32_t h2[kBins];
   uint32_t h3[1 << kL3Bits];
@@ -2065,6 +2065,38 @@ cudaError_t mark(const cudaEvent_t* marks, int i, cudaStream_t s) {
   return (marks && marks[i]) ? cudaEventRecordWithFlags(marks[i], s, cudaEventRecordExternal) : cudaSuccess;
 }
 
+size_t small_smem(int64_t d) {
+  const int64_t per = ((d + 31) / 32 + kSmallCtas - 1) / kSmallCtas;
+  return sizeof(SmallShared) + 2 * (size_t)per * sizeof(uint32_t);
+}
+
+// Whether the current device can hold the cluster of k_select_small (asked once per device).  16 CTAs
+// that take an SM each are twice the portable size: a partition of the device, or one with fewer SMs
+// in use per processing cluster, may not place them, and short vectors are then selected by the kernels
+// for long ones.
+bool small_cluster_fits() {
+  static std::mutex mu;
+  static std::unordered_map<int, bool> fits;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  std::lock_guard<std::mutex> lock(mu);
+  const auto it = fits.find(dev);
+  if (it != fits.end()) return it->second;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kSmallCtas);
+  cfg.blockDim = dim3(kSmallThreads);
+  cfg.dynamicSmemBytes = small_smem(kSmallMaxDim);
+  int n = 0;
+  cudaError_t e = cudaFuncSetAttribute(k_select_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_select_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k_select_small, &cfg);
+  if (e != cudaSuccess) cudaGetLastError();  // not an error of this call
+  return fits.emplace(dev, e == cudaSuccess && n > 0).first->second;
+}
+
+bool selects_small(int64_t d) { return d <= kSmallMaxDim && small_cluster_fits(); }
+
 // Histograms and state (adjacent) and, unless the selection goes by one cluster, both bitmaps
 // (adjacent) back to zero.
 cudaError_t clear_selection(const Workspace& w, int64_t d, cudaStream_t s) {
@@ -2085,8 +2117,7 @@ cudaError_t launch_query_bits(const QueryParams& p, const Workspace& w, cudaStre
 // Levels 2 and 3 and the ordered output by one cluster; `picked`: see k_select_small.
 cudaError_t select_small(const float* src, int vec, uint32_t kmask, const uint32_t* hist1, const SelectState* st,
                          int picked, int64_t d, int64_t k, int64_t* idx_out, cudaStream_t s) {
-  const int64_t per = ((d + 31) / 32 + kSmallCtas - 1) / kSmallCtas;
-  const size_t smem = sizeof(SmallShared) + 2 * (size_t)per * sizeof(uint32_t);
+  const size_t smem = small_smem(d);
   cudaError_t e = cudaFuncSetAttribute(k_select_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_select_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
