@@ -624,7 +624,8 @@ template <int WT, bool POW2>
 cudaError_t launch_staged_t(const InsertParams& p, int W, cudaStream_t s) {
   auto kern = k_insert_staged<WT, POW2>;
   const size_t smem = (size_t)p.c * WT * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the limit that every call sets: another thread's launch may stand between this call's setting and launch
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStagedSmemBytes);
   if (e != cudaSuccess) return e;
   // about two CTAs per SM over all (row, worker tile) pairs, at least one chunk
   const int tiles = (p.j1 - p.j0) * (W / WT);

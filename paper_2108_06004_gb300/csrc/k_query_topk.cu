@@ -1796,7 +1796,8 @@ cudaError_t launch_query_bits_r(const QueryParams& p, uint32_t* words, cudaStrea
   launch(k_pbits, (int)(warps < cap ? warps : cap), kBlock, s, p.T, p.c, nwords, p.st, words);
   auto kern = p.keys ? k_query_bits<R, true> : k_query_bits<R, false>;
   const size_t smem = (size_t)nwords * 2 * sizeof(uint32_t);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the limit that every call sets: another thread's launch may stand between this call's setting and launch
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBitsBytes);
   if (e != cudaSuccess) return e;
   const int64_t need = ((p.d + 3) / 4 + kBitsBlock - 1) / kBitsBlock;
   const int grid = (int)(need < device_info().sms ? (need < 1 ? 1 : need) : device_info().sms);
@@ -2117,14 +2118,14 @@ cudaError_t launch_query_bits(const QueryParams& p, const Workspace& w, cudaStre
 // Levels 2 and 3 and the ordered output by one cluster; `picked`: see k_select_small.
 cudaError_t select_small(const float* src, int vec, uint32_t kmask, const uint32_t* hist1, const SelectState* st,
                          int picked, int64_t d, int64_t k, int64_t* idx_out, cudaStream_t s) {
-  const size_t smem = small_smem(d);
   cudaError_t e = cudaFuncSetAttribute(k_select_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_select_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_select_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)small_smem(kSmallMaxDim));
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kSmallCtas);
   cfg.blockDim = dim3(kSmallThreads);
-  cfg.dynamicSmemBytes = smem;
+  cfg.dynamicSmemBytes = small_smem(d);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
