@@ -30,8 +30,8 @@
 //   k_bm_count    per block of 65536 coordinates: bits set in each bitmap
 //   k_scan        one CTA: exclusive prefix sums over the blocks
 //   k_bm_write    every block writes its selected indices at their final positions
-// Up to d = 1.5 * 2^20 one launch of k_select_small replaces k_cand .. k_bm_write, where the device can
-// hold its cluster.
+// Up to d = 1.5 * 2^20 (large k: 819,200) one launch of k_select_small replaces k_cand .. k_bm_write, where
+// the device can hold its cluster.
 // With the fixed scratch (gs_query_topk_noalloc), which cannot hold candidate lists, the
 // levels 2 and 3 and the final selection read est in full passes (k_hist, k_count, k_write).
 #include <cmath>
@@ -1334,11 +1334,16 @@ __global__ void __launch_bounds__(kBmThreads) k_bm_write(const uint32_t* __restr
 // cluster barriers stand where the kernels were.  Query and selection in us, k = d/1000 (d/100), six
 // kernels / one cluster: d = 100k 35.2 / 22.0 (37.1 / 22.1), 300k 39.1 / 25.9 (42.4 / 28.2), 2^20 50.1 / 39.7
 // (53.7 / 47.2), 2M 68.6 / 64.4 (72.2 / 75.7), 4M 108 / 112 (113 / 171): beyond 1.5 * 2^20 the 136 idle SMs
-// cost more than the launches.
+// cost more than the launches.  Writing many indices from 16 CTAs costs more than the launches as well,
+// from about 819,200 coordinates on: k = d/50, d/10, d/2: d = 420k 40.9 / 32.1, 46.3 / 35.2, 59.5 / 43.0,
+// 800k 49.4 / 45.7, 54.4 / 51.7, 68.1 / 65.3, 2^20 51.8 / 49.1, 57.9 / 58.4, 71.8 / 75.8, 1.5 * 2^20
+// 58.7 / 62.4, 67.0 / 80.1, 79.2 / 104.  Keys that are all equal, which overflow the lists, follow the same
+// line (k = d/10, 800k 98.6 / 92.4, 2^20 109 / 128).
 constexpr int kSmallCtas = 16;
 constexpr int kSmallThreads = 1024;
 constexpr int kSmallList = 16384;                   // candidates kept per CTA
 constexpr int64_t kSmallMaxDim = int64_t(3) << 19;  // 3072 bitmap words per CTA
+constexpr int64_t kSmallAnyK = int64_t(25) << 15;   // up to this length for any k, beyond for k <= d/100
 
 struct SmallShared {
   uint32_t h2[kBins];
@@ -2096,14 +2101,16 @@ bool small_cluster_fits() {
   return fits.emplace(dev, e == cudaSuccess && n > 0).first->second;
 }
 
-bool selects_small(int64_t d) { return d <= kSmallMaxDim && small_cluster_fits(); }
+bool selects_small(int64_t d, int64_t k) {
+  return d <= kSmallMaxDim && (d <= kSmallAnyK || k <= d / 100) && small_cluster_fits();
+}
 
 // Histograms and state (adjacent) and, unless the selection goes by one cluster, both bitmaps
 // (adjacent) back to zero.
-cudaError_t clear_selection(const Workspace& w, int64_t d, cudaStream_t s) {
+cudaError_t clear_selection(const Workspace& w, int64_t d, int64_t k, cudaStream_t s) {
   const size_t head = (size_t)(reinterpret_cast<char*>(w.st + 1) - reinterpret_cast<char*>(w.hist));
   cudaError_t err = cudaMemsetAsync(w.hist, 0, head, s);
-  if (err == cudaSuccess && !selects_small(d))
+  if (err == cudaSuccess && !selects_small(d, k))
     err = cudaMemsetAsync(w.gt_bm, 0, (size_t)(reinterpret_cast<char*>(w.blk) - reinterpret_cast<char*>(w.gt_bm)), s);
   return err;
 }
@@ -2162,7 +2169,7 @@ cudaError_t launch_query_topk(const float* merged, const HashCoeffs& h, int r, u
                               void* workspace, cudaStream_t s, const RowStrides& slow, const cudaEvent_t* marks) {
   Workspace w = carve(workspace, d);
   float* est = est_out ? est_out : w.est;
-  cudaError_t err = clear_selection(w, d, s);
+  cudaError_t err = clear_selection(w, d, k, s);
   if (err != cudaSuccess) return err;
   if ((err = mark(marks, 0, s)) != cudaSuccess) return err;
 
@@ -2170,7 +2177,7 @@ cudaError_t launch_query_topk(const float* merged, const HashCoeffs& h, int r, u
   // rows are pruned only while the estimate stays internal: a caller's est_out gets every value
   const uint32_t j_target = sample_rank(d, k);
   qp.prune = (!est_out && can_prune(r, c, d) && j_target > 0) ? 1 : 0;
-  qp.pick = (qp.prune || !selects_small(d)) ? 1 : 0;  // k_repair needs the pick, and so do many CTAs
+  qp.pick = (qp.prune || !selects_small(d, k)) ? 1 : 0;  // k_repair needs the pick, and so do many CTAs
   if (qp.prune) {
     using T = SampleTable<1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16>;
     if ((err = T::table[r - 1](qp, w.hist + 4 * kBins, j_target, s)) != cudaSuccess) return err;
@@ -2185,7 +2192,7 @@ cudaError_t launch_query_topk(const float* merged, const HashCoeffs& h, int r, u
     if ((err = T::table[r - 1](qp, w.hist + 3 * kBins, s)) != cudaSuccess) return err;
   }
   if ((err = mark(marks, 1, s)) != cudaSuccess) return err;
-  if (selects_small(d)) err = select_small(est, qp.vec, 0x7FFFFFFFu, w.hist, w.st, qp.pick, d, k, idx_out, s);
+  if (selects_small(d, k)) err = select_small(est, qp.vec, 0x7FFFFFFFu, w.hist, w.st, qp.pick, d, k, idx_out, s);
   else err = select_from_keys(w, est, qp.vec, 0x7FFFFFFFu, d, k, idx_out, s);
   return err != cudaSuccess ? err : mark(marks, 2, s);
 }
@@ -2211,7 +2218,7 @@ cudaError_t launch_query_heavymix(const float* merged, const HashCoeffs& h, int 
   double* sumsq = reinterpret_cast<double*>(extra + align256((size_t)d * sizeof(uint32_t)));
   double* theta = sumsq + GS_MAX_ROWS;
   float* est = est_out ? est_out : w.est;
-  cudaError_t err = clear_selection(w, d, s);
+  cudaError_t err = clear_selection(w, d, k, s);
   if (err == cudaSuccess) err = cudaMemsetAsync(sumsq, 0, 256, s);
   if (err == cudaSuccess) err = mark(marks, 0, s);
   if (err != cudaSuccess) return err;
@@ -2225,7 +2232,7 @@ cudaError_t launch_query_heavymix(const float* merged, const HashCoeffs& h, int 
   // the query stores each coordinate's composite key and picks on their level-1 histogram
   QueryParams qp = make_query_params(merged, h, r, c, d, k, est, w.hist, w.st);
   qp.prune = prune;
-  qp.pick = (prune || !selects_small(d)) ? 1 : 0;
+  qp.pick = (prune || !selects_small(d, k)) ? 1 : 0;
   qp.keys = keys;
   qp.theta = theta;
   qp.fill_seed = fill_seed;
@@ -2234,7 +2241,7 @@ cudaError_t launch_query_heavymix(const float* merged, const HashCoeffs& h, int 
   if (err != cudaSuccess) return err;
   if ((err = mark(marks, 1, s)) != cudaSuccess) return err;
   const float* src = reinterpret_cast<const float*>(keys);
-  if (selects_small(d)) err = select_small(src, 1, 0xFFFFFFFFu, w.hist, w.st, qp.pick, d, k, idx_out, s);
+  if (selects_small(d, k)) err = select_small(src, 1, 0xFFFFFFFFu, w.hist, w.st, qp.pick, d, k, idx_out, s);
   else err = select_from_keys(w, src, 1, 0xFFFFFFFFu, d, k, idx_out, s);
   return err != cudaSuccess ? err : mark(marks, 2, s);
 }
@@ -2338,9 +2345,9 @@ cudaError_t launch_query_topk_noalloc(const float* merged, const HashCoeffs& h, 
   if (err != cudaSuccess) return err;
 
   QueryParams qp = make_query_params(merged, h, r, c, d, k, est_out, hist, st);
-  qp.pick = selects_small(d) ? 0 : 1;
+  qp.pick = selects_small(d, k) ? 0 : 1;
   if ((err = launch_query(qp, slow, s)) != cudaSuccess) return err;
-  if (selects_small(d)) return select_small(est_out, qp.vec, 0x7FFFFFFFu, hist, st, 0, d, k, idx_out, s);
+  if (selects_small(d, k)) return select_small(est_out, qp.vec, 0x7FFFFFFFu, hist, st, 0, d, k, idx_out, s);
   const int hgrid = persistent_grid(k_hist, (d + 3) / 4 / kU, kBlock);
   launch(k_hist, hgrid, kBlock, s, est_out, d, qp.vec, st, hist + kBins, kL2Shift, 11, 1);
   launch(k_hist, hgrid, kBlock, s, est_out, d, qp.vec, st, hist + 2 * kBins, 0, kL3Bits, 2);
