@@ -183,10 +183,60 @@ gs_status check_vec(const void* p, const char* name) {
 
 cudaStream_t as_stream(gs_stream s) { return reinterpret_cast<cudaStream_t>(s); }
 
-// Inserts the vectors e[0..nw) of length d by chains into rows [j0, r) of the table whose cell
-// (row j, bucket b) is cells[(j * c + b) * pitch]; W: workers of a cell written.
-gs_status insert_chains(const gs_sketch* sk, float* cells, int pitch, int W, int j0, const float* const* e, int nw,
-                        int64_t d, cudaStream_t s) {
+// The chains of rows [j0, r) for vectors of length d (c a power of two), and the cell updates that they
+// save for a coordinate, of one per row.
+struct Chains {
+  int j0 = 0;
+  gs::ChainShape row[GS_MAX_ROWS];
+  double saved = 0.0;
+};
+
+Chains choose_chains(const gs_sketch* sk, int j0, int64_t d) {
+  Chains ch;
+  ch.j0 = j0;
+  // Chains as long as two waves of 1536 threads per SM allow, and 32 at most: longer ones leave too few
+  // CTAs to even out the last wave (d = 25,557,032, 4 rows: 16, 32, 64 steps all within 1 %).  Up to 12 steps
+  // one wave is enough, since short chains save little: single inserts, one wave / two, r = 3, d = 230k, c = 2^14
+  // 5.2 / 7.5 us, r = 5, d = 100k 4.0 / 5.2; but r = 5, d = 1.4M (30 steps / 15) 16.8 / 14.7.
+  const int64_t wave = (int64_t)gs::device_info().sms * 1536, work = (sk->r - j0) * d;
+  const int64_t max_steps =
+      std::min<int64_t>(32, std::max({std::min<int64_t>(12, work / wave), work / (2 * wave), int64_t(1)}));
+  for (int j = j0; j < sk->r; ++j) {
+    ch.row[j - j0] = gs::choose_chain(sk->rotation[j], d, kMinStride, max_steps);
+    ch.saved += 1.0 - ch.row[j - j0].flushes;
+  }
+  return ch;
+}
+
+// A table beyond this does not stay in L2: reductions into all its rows at once miss, while the chains take
+// one row after the other.
+constexpr size_t kLargeTable = size_t(96) << 20;
+constexpr int64_t kShortVector = int64_t(5) << 14;
+
+size_t group_table_bytes(const gs_sketch* sk) { return (size_t)sk->r * sk->c * sk->W * sizeof(float); }
+
+// Whether to insert already accumulated vectors by these chains (of all rows) rather than by one reduction
+// per coordinate and row; W: workers of a cell written.  Chained, a row reads the vectors once, with 4-byte
+// loads, and saves updates; without enough of them to save it is the slower kernel, except that its rows run
+// side by side, which wins where the vectors are short.  Chained by direct time where chains save 0.1, 0.2,
+// 0.3, 0.4, 0.5 of the updates (d >= 2^16, medians over 780 shapes): one vector 0.96, 0.95, 0.77, 0.74, 0.59.
+// Chained minus direct in a sketched-state step, us: 8 workers +2.0, 0.0, -1.0, -1.5, -1.1, 16 workers +1.7,
+// +2.7, +5.4, +3.6, +2.0.
+bool chains_pay(const gs_sketch* sk, const Chains& ch, int W, int64_t d) {
+  const bool large = group_table_bytes(sk) > kLargeTable;
+  if (W == 16) return ch.saved > 0.55 * sk->r || (large && d < kShortVector);
+  if (large || ch.saved > 0.15 * sk->r) return true;
+  // few cells: the updates of one row collide whether chained or not (c = 256, d = 33k, r = 1: 9.2 us
+  // chained, 6.4 not), those of several rows less when they run side by side (r = 2, d = 160k: 18, 22 us)
+  if (sk->r == 1) return d < kShortVector && d < 32 * (int64_t)sk->c;
+  return d < kShortVector || sk->c <= 512;
+}
+
+// Inserts the vectors e[0..nw) of length d along these chains into the table whose cell (row j, bucket b)
+// is cells[(j * c + b) * pitch]; W: workers of a cell written.
+gs_status insert_chains(const gs_sketch* sk, const Chains& ch, float* cells, int pitch, int W, const float* const* e,
+                        int nw, int64_t d, cudaStream_t s) {
+  const int j0 = ch.j0;
   if (j0 >= sk->r) return GS_OK;
   gs::ChainParams p;
   std::memset(&p, 0, sizeof(p));
@@ -197,34 +247,31 @@ gs_status insert_chains(const gs_sketch* sk, float* cells, int pitch, int W, int
   p.pitch = pitch;
   p.nrows = sk->r - j0;
   p.resident = (size_t)d * nw * sizeof(float) <= kResidentBytes ? 1 : 0;
-  // Chains as long as two waves of 1536 threads per SM allow, and 32 at most: longer ones leave
-  // too few CTAs to even out the last wave (d = 25,557,032, 4 rows: 16, 32, 64 steps all within 1 %).
-  const int64_t lanes = (int64_t)gs::device_info().sms * 1536 * 2;
-  const int64_t max_steps = std::min<int64_t>(32, std::max<int64_t>(1, p.nrows * d / lanes));
   for (int j = j0; j < sk->r; ++j) {
     gs::ChainRow& row = p.row[j - j0];
-    const gs::ChainShape ch = gs::choose_chain(sk->rotation[j], d, kMinStride, max_steps);
+    const gs::ChainShape& shape = ch.row[j - j0];
     row.a8 = 8 * sk->h.a[j];
     row.b8 = 8 * sk->h.b[j];
     row.a28 = 8 * sk->h.a2[j];
     row.b28 = 8 * sk->h.b2[j];
-    row.sa8 = 8 * gs::mulmod61(sk->h.a[j], (uint64_t)ch.stride);
-    row.sa28 = 8 * gs::mulmod61(sk->h.a2[j], (uint64_t)ch.stride);
+    row.sa8 = 8 * gs::mulmod61(sk->h.a[j], (uint64_t)shape.stride);
+    row.sa28 = 8 * gs::mulmod61(sk->h.a2[j], (uint64_t)shape.stride);
     row.cells = cells + (size_t)j * sk->c * pitch;
-    row.stride = ch.stride;
-    row.steps = ch.steps;
+    row.stride = shape.stride;
+    row.steps = shape.steps;
   }
   const cudaError_t err = gs::launch_insert_chain(p, W, s);
   if (err != cudaSuccess) return cuda_fail(err, "chained insert launch");
   return GS_OK;
 }
 
-// What the accumulate pass of a group inserts (c a power of two): rows [0, rows), along chains
-// that serve row 0 (walk) or one reduction per coordinate and row; the other rows go by
-// insert_chains, which reads the error vectors once more per row.
+// What the accumulate pass of a group inserts (c a power of two): rows [0, rows), along chains that
+// serve row 0 (walk) or one reduction per coordinate and row.  The other rows go along chains, which read
+// the error vectors once more per row, or (chains false) by reductions in further passes.
 struct MainPass {
   int rows;
   bool walk;
+  bool chains;
 };
 
 // Insert phase in ms, r = 5: all rows directly / none, all by insert_chains / walking with W/2 rows
@@ -238,16 +285,42 @@ struct MainPass {
 //   16 workers, 7 x 2^20 cells (32 MiB a row and group), d = 138M: 23.5 / 17.1 / 16.6 with one row
 //   16 workers, 5 x 2^21 (64 MiB a row), d = 83M: 10.6 / 9.1 / 9.3 with one row
 // Up to 2^20 updates (5 us of reductions) a second launch costs more than it saves (d = 100k, W = 4,
-// r = 5: 12 us direct, 14 us in two launches).  Gradients read from host memory are bound by the link
-// to the host, under which the direct reductions cost nothing.
-MainPass main_pass(const gs_sketch* sk, int64_t d, bool remote) {
-  if (d * sk->r <= kFewUpdates) return {sk->r, false};
-  if (remote) return {sk->rows_per_pass, false};
-  const size_t row_bytes = (size_t)sk->c * sk->W * sizeof(float);
-  if (d < kWalkMinDim) return {sk->W == 16 ? sk->rows_per_pass : 0, false};
-  const int rows = sk->W == 16 ? sk->r : std::max(1, sk->W / 2);
-  const int rows_in_l2 = (int)std::min<size_t>(kPassBudget / row_bytes, (size_t)sk->r);
-  return {std::min(rows, rows_in_l2), rows_in_l2 > 0};
+// r = 5: 12 us direct, 14 us in two launches).  Between there and the walk's length, chains have to save
+// more updates than a launch costs (base), beyond what reading the vectors again costs (reread, per row)
+// and what hides under the accumulate pass (hidden, in rows).  The lines are those with the least loss over
+// 805 shapes (r 1 to 16, c 2^10 to 2^21, d 66k to 3.9M): always chained, 132 of them are more than 4 % slower
+// than by reductions alone, by up to 78 %; with the lines 16, by up to 21 %.  Direct / chained: W = 4, r = 16,
+// c = 2^17, d = 130k 12.5 / 19.5 us; W = 8, r = 9, c = 2^17, d = 130k 13.7 / 17.8; W = 8, r = 1, c = 2^17, d = 2.5M
+// 72.7 / 81.2.  A single row of 8 or 16 workers walks no faster than it goes by reductions (W = 8, d = 6M,
+// c = 2^14: 177 / 198 us).
+// Gradients read from host memory are bound by the link to the host, under which the direct reductions
+// cost nothing.
+MainPass main_pass(const gs_sketch* sk, int64_t d, bool remote, Chains& rest) {
+  const int r = sk->r, W = sk->W;
+  const MainPass direct = {sk->rows_per_pass, false, false};
+  if (d * r <= kFewUpdates) return {r, false, false};
+  if (d >= kWalkMinDim && !remote) {
+    const size_t row_bytes = (size_t)sk->c * W * sizeof(float);
+    const int rows_in_l2 = (int)std::min<size_t>(kPassBudget / row_bytes, (size_t)r);
+    if (r == 1 && W >= 8 && rows_in_l2 == 1) return direct;
+    const int rows = std::min(W == 16 ? r : std::max(1, W / 2), rows_in_l2);
+    rest = choose_chains(sk, rows, d);
+    return {rows, rows_in_l2 > 0, true};
+  }
+  const int rows = remote || W == 16 ? sk->rows_per_pass : 0;
+  rest = choose_chains(sk, rows, d);
+  if (remote) return rest.saved > (W == 16 ? 0.55 : 0.15) * (r - rows) ? MainPass{rows, false, true} : direct;
+  struct Line {
+    double reread, hidden, base;
+  };
+  const Line line = W == 16                           ? Line{0.0, 0.0, 300e3}
+                    : group_table_bytes(sk) > kLargeTable ? Line{0.0, 0.0, 25e3}
+                    : W == 8                              ? Line{0.2, 1.4, 0.0}
+                    : W == 4                              ? Line{0.15, 0.5, 550e3}
+                    : W == 2                              ? Line{0.15, 0.0, 200e3}
+                                                          : Line{0.15, 0.0, 100e3};
+  const bool pays = (double)d * (rest.saved - line.reread * (r - rows) - line.hidden) > line.base;
+  return pays ? MainPass{rows, false, true} : direct;
 }
 
 gs_status accumulate_insert_impl(gs_sketch* sk, int32_t first, int32_t n, float* const* m,
@@ -255,6 +328,9 @@ gs_status accumulate_insert_impl(gs_sketch* sk, int32_t first, int32_t n, float*
                                  cudaStream_t s, bool remote = false) {
   const int W = sk->W;
   const int end = first + n;
+  const bool pow2 = !sk->rotation.empty();
+  Chains rest;
+  const MainPass mp = pow2 ? main_pass(sk, d, remote, rest) : MainPass{0, false, false};
   for (int grp = first / W; grp * W < end; ++grp) {
     gs::InsertParams p;
     std::memset(&p, 0, sizeof(p));
@@ -277,8 +353,7 @@ gs_status accumulate_insert_impl(gs_sketch* sk, int32_t first, int32_t n, float*
     p.cinv = gs::bucket_inverse((uint32_t)sk->c);
     p.rho = rho;
     p.h = sk->h;
-    if (!sk->rotation.empty()) {
-      const MainPass mp = main_pass(sk, d, remote);
+    if (pow2 && (mp.chains || mp.rows == sk->r)) {
       p.j1 = mp.rows;
       cudaError_t err;
       if (mp.walk) {
@@ -291,7 +366,7 @@ gs_status accumulate_insert_impl(gs_sketch* sk, int32_t first, int32_t n, float*
         err = gs::launch_accumulate_insert(p, W, true, vec, s);
       }
       if (err != cudaSuccess) return cuda_fail(err, "accumulate_insert launch");
-      GS_TRY(insert_chains(sk, p.table, W, W, p.j1, p.e, nw, d, s));
+      if (mp.chains) GS_TRY(insert_chains(sk, rest, p.table, W, W, p.e, nw, d, s));
       continue;
     }
     // first pass: accumulate and insert the first slice; later passes insert the remaining
@@ -312,6 +387,9 @@ gs_status accumulate_insert_impl(gs_sketch* sk, int32_t first, int32_t n, float*
 // Insert the vectors vec[p] (no accumulation) into the worker tables, all groups and passes.
 gs_status insert_all_impl(gs_sketch* sk, const float* const* vec, int64_t d, cudaStream_t s) {
   const int W = sk->W;
+  Chains ch;
+  if (!sk->rotation.empty()) ch = choose_chains(sk, 0, d);
+  const bool chained = !sk->rotation.empty() && chains_pay(sk, ch, W, d);
   for (int grp = 0; grp * W < sk->workers; ++grp) {
     gs::InsertParams p;
     std::memset(&p, 0, sizeof(p));
@@ -330,8 +408,8 @@ gs_status insert_all_impl(gs_sketch* sk, const float* const* vec, int64_t d, cud
     p.cmask = (uint32_t)sk->c - 1;
     p.cinv = gs::bucket_inverse((uint32_t)sk->c);
     p.h = sk->h;
-    if (!sk->rotation.empty()) {
-      GS_TRY(insert_chains(sk, p.table, W, W, 0, p.e, nw, d, s));
+    if (chained) {
+      GS_TRY(insert_chains(sk, ch, p.table, W, W, p.e, nw, d, s));
       continue;
     }
     p.evict = sk->rows_per_pass < sk->r;
@@ -839,8 +917,10 @@ gs_status gs_sketch_insert(gs_sketch* sk, int32_t worker, const float* vec, int6
   if (worker < 0 || worker >= sk->workers) return fail(GS_ERR_INVALID_ARG, "worker out of range");
   const int W = sk->W;
   float* const table = sk->tables + (size_t)(worker / W) * sk->r * sk->c * W;
-  if (!sk->rotation.empty())
-    return insert_chains(sk, table + worker % W, W, 1, 0, &vec, 1, d, as_stream(stream));
+  if (!sk->rotation.empty()) {
+    const Chains ch = choose_chains(sk, 0, d);
+    if (chains_pay(sk, ch, 1, d)) return insert_chains(sk, ch, table + worker % W, W, 1, &vec, 1, d, as_stream(stream));
+  }
   gs::InsertParams p;
   std::memset(&p, 0, sizeof(p));
   p.e[0] = const_cast<float*>(vec);

@@ -345,7 +345,8 @@ __global__ void __launch_bounds__(kBlock, 3) k_accumulate_chain(const __grid_con
     if (cur[t] != kNoCell) red_lane<N>(crow + (size_t)cur[t] * W, acc[t], pol_table);
 }
 
-// Insert one vector (prm.e[0]) into lane prm.lane of a W-wide group table, c not a power of two.
+// Insert one vector (prm.e[0]) into lane prm.lane of a W-wide group table.
+template <bool POW2>
 __global__ void __launch_bounds__(kBlock) k_insert_lane(const __grid_constant__ InsertParams prm, int W) {
   grid_begin();
   const int64_t d = prm.d;
@@ -367,7 +368,7 @@ __global__ void __launch_bounds__(kBlock) k_insert_lane(const __grid_constant__ 
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
         if (t < tmax) {
-          const uint32_t bk = bucket_of<false>(x, prm.c, prm.cmask, prm.cinv);
+          const uint32_t bk = bucket_of<POW2>(x, prm.c, prm.cmask, prm.cinv);
           red_add_f32(row + (size_t)bk * W, apply_sign(ev[t], signbit_of(y)));
           x = step61(x, a);
           y = step61(y, a2);
@@ -560,10 +561,7 @@ cudaError_t launch_ai_t(const InsertParams& p, cudaStream_t s) {
 
 template <int W, bool ACC>
 cudaError_t launch_ai_w(const InsertParams& p, bool vec, cudaStream_t s) {
-  // without accumulation only c that are not powers of two come here: the others go by chains
-  if constexpr (ACC) {
-    if (is_pow2(p.c)) return vec ? launch_ai_t<W, ACC, true, true>(p, s) : launch_ai_t<W, ACC, false, true>(p, s);
-  }
+  if (is_pow2(p.c)) return vec ? launch_ai_t<W, ACC, true, true>(p, s) : launch_ai_t<W, ACC, false, true>(p, s);
   return vec ? launch_ai_t<W, ACC, true, false>(p, s) : launch_ai_t<W, ACC, false, false>(p, s);
 }
 
@@ -714,7 +712,8 @@ cudaError_t launch_insert_chain(ChainParams& p, int W, cudaStream_t s) {
 }
 
 cudaError_t launch_insert_lane(const InsertParams& p, int W, cudaStream_t s) {
-  launch(k_insert_lane, grid_for(k_insert_lane, (p.d + 3) / 4, kBlock), kBlock, s, p, W);
+  auto kern = is_pow2(p.c) ? k_insert_lane<true> : k_insert_lane<false>;
+  launch(kern, grid_for(kern, (p.d + 3) / 4, kBlock), kBlock, s, p, W);
   return cudaGetLastError();
 }
 
