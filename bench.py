@@ -449,7 +449,8 @@ def launches_per_step(run: Runner, variant: str) -> int:
     bits = w.d >= PRUNE_MIN_DIM and query_classifies(w.r, w.c)
     select = 1 if w.d <= 3 << 19 else 6               # one cluster up to 1.5 * 2^20 coordinates
     if variant == "heavymix":
-        query = 3 + int(bits) + select                # sumsq, theta, query (with the keys) + selection
+        # sumsq, theta, query (with the keys) + selection; k_query behind it where few may settle
+        query = 3 + int(bits) + int(bits and w.k > w.c // 8 and w.r < 16) + select
     else:
         # query + selection (+ sample and repair check, + the cell classes)
         query = 1 + select + (2 + int(bits) if prunes else 0)

@@ -205,8 +205,8 @@ gs_status gs_query_heavymix_workspace_size(int64_t d, int64_t k, size_t* bytes);
  * With est_out NULL, d >= 2^22, r >= 3 and c a power of two, rows are skipped as in
  * gs_query_topk with t = sqrt(l2sq / k) (rounded down to a bin edge): a coordinate that stops
  * has est^2 below the threshold, so it can only enter through the fill, and its estimate is
- * left in the workspace as the marker described there; idx_out is the same as without
- * skipping. */
+ * left in the workspace as the marker described there (g = n also where the classes fit but
+ * settle few coordinates); idx_out is the same as without skipping. */
 gs_status gs_query_heavymix(const gs_sketch* sketch, int64_t d, int64_t k, uint64_t fill_seed,
                             int64_t* idx_out, float* est_out, double* l2sq_out, void* workspace,
                             size_t workspace_bytes, gs_stream stream);

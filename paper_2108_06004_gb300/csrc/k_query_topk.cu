@@ -71,6 +71,7 @@ struct SelectState {
                        // query, before k_query, by k_qsample or k_heavy_theta
   uint32_t done_r;     // CTAs finished in k_repair
   uint32_t done_s;     // CTAs finished in k_qsample
+  uint32_t open;       // HEAVYMIX: k_query_bits left the whole query to k_query
 };
 
 inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -247,6 +248,8 @@ struct QueryParams {
   int32_t vec;        // est 16-byte aligned
   int32_t pick;       // the last CTA picks the level-1 bin from the histogram of the keys
   int32_t prune;      // skip rows below st->prune_key (estimate internal to the workspace)
+  int32_t if_open;    // HEAVYMIX: k_query is launched behind k_query_bits and runs only where that kernel left the
+                      // query to it (st->open)
   uint32_t* keys;     // HEAVYMIX: also store each coordinate's composite key here, and build the
                       // level-1 histogram (and pick) on those keys instead of |est|
   const double* theta;  // HEAVYMIX: the threshold l2sq / k of H
@@ -325,6 +328,7 @@ __device__ __forceinline__ void store_est(const QueryParams& prm, int64_t i0, in
 template <int R, bool HM = false>
 __global__ void __launch_bounds__(kBlock, R <= 7 ? 4 : 1) k_query(const __grid_constant__ QueryParams prm) {
   grid_begin();
+  if (HM && prm.if_open && __ldcg(&prm.st->open) == 0u) return;
   __shared__ uint32_t sh[kBins];
   for (int b = threadIdx.x; b < kBins; b += blockDim.x) sh[b] = 0;
   __syncthreads();
@@ -642,22 +646,38 @@ __global__ void __launch_bounds__(kBlock, R <= 7 ? 3 : 2) k_query_walk(const __g
 // k_query_bits looks them up instead of reading those cells from L2.  A coordinate that settles
 // within the first f rows then reads no cell at all; one that examines later rows reads those
 // cells as k_query does; one that does not settle reads every cell for its full median.  The rows
-// examined, the stops and the estimates are the same as k_query's.
+// examined, the stops and the estimates are the same as k_query's, for tables without NaN (a NaN cell
+// counts on the side of its sign bit here and on neither there).
 //
 // The kernel sorts its coordinates by the work that they need, so that warps stay full.
 //   1. f rows settle a coordinate exactly when all f cells are inside, whatever the signs: four
 //      coordinates per lane, only the buckets of the first f rows, whose hash comes from a form
 //      that needs few instructions (rot_add).  The others are queued, per warp.
-//   2. With one cell of the first f outside, the next row settles a coordinate exactly when its
-//      cell is inside, again whatever the signs: 32 such coordinates at a time, one per lane, one
-//      bucket and one cell read each.
+//   2. With one cell of the first f outside, the next row settles a coordinate when its cell is
+//      inside, again whatever the signs: 32 such coordinates at a time, one per lane, one bucket and
+//      one cell read each.
 //   3. What is left is resolved from its signs and all further rows, 32 coordinates at a time.
 // Integer instructions bound it.  d = 25,557,032, r = 5, c = 2^18: 0.098 ms, and 0.110 in HEAVYMIX
 // mode (which evaluates the fill order of every coordinate); one kernel for all coordinates, four per
 // lane, took 0.267, and 0.344 with k_query in HEAVYMIX mode.  Part 3 without part 2 takes 0.145.
+//
+// The sorting pays while parts 1 and 2 settle enough coordinates; where most are left for part 3 (a large k,
+// many rows, few columns: the prune key lies within the cells' noise), evaluating every row of four
+// coordinates per lane from the start is the better order (query_quads), and a CTA takes it when the bits
+// say that more than kMostlyOpen of them will be left.  Query with its selection in us, sorted / quads,
+// d = 25.6M: r = 7, c = 2^16, k = d/1000, d/100, d/30, d/10 (shares left 0.19, 0.52, 0.71, 0.80) 277 / 440,
+// 456 / 478, 599 / 533, 652 / 551; r = 16, c = 2^14, k = d/1000 (0.97) 1450 / 1127.  The line is the one with the
+// least loss over 610 shapes (r 3 to 16, c 2^10 to 2^18, k d/10000 to d/3).  With many rows and few cells inside,
+// nearly every coordinate reads every cell; the quads' registers spill, and one coordinate per lane is the
+// faster order again where the cells come from L2 (r = 16, k = d/3, 0.22 of the cells inside: c = 2^14 1781 /
+// 1951, c = 2^16 1696 / 1990, but c = 2^10 1566 / 1270).
 constexpr uint32_t kBitsBytes = 192u << 10;   // dynamic shared memory for the bits
 
 constexpr int kBitsBlock = 1024;              // one CTA of 32 warps per SM
+constexpr float kMostlyOpen = 0.55f;          // share left for part 3 from which quads are faster
+// ... and in HEAVYMIX mode k_query, which reads the cells from the start: where its threshold leaves most
+// coordinates open, they need every cell.  k_query has more to spill for many rows.
+__host__ __device__ constexpr float heavy_open(int r) { return r < 8 ? 0.6f : r < 11 ? 0.75f : r < 16 ? 0.87f : 1.f; }
 // Queue entries per warp.  Queue 2 grows from the front, queue 3 from the back; each keeps at most
 // 31 entries from one grid stride to the next, which adds at most 128.
 constexpr int kQueue = 192;
@@ -734,6 +754,114 @@ __device__ __forceinline__ float resolve(const QueryParams& prm, const uint32_t*
   return median_of<R>(v);
 }
 
+// The share of the coordinates that parts 1 and 2 leave open, p of the cells being inside.
+template <int R>
+__device__ __forceinline__ float left_open(float p) {
+  constexpr int kF = R / 2 + 1;
+  float few = 1.f;  // p^(kF - 1)
+#pragma unroll
+  for (int j = 1; j < kF; ++j) few *= p;
+  return 1.f - few * p - (kF + 1 < R ? kF * few * (1.f - p) * p : 0.f);
+}
+
+// The even bits of the result are the low 16 bits of x.
+__device__ __forceinline__ uint32_t spread_bits(uint32_t x) {
+  x &= 0xFFFFu;
+  x = (x | (x << 8)) & 0x00FF00FFu;
+  x = (x | (x << 4)) & 0x0F0F0F0Fu;
+  x = (x | (x << 2)) & 0x33333333u;
+  return (x | (x << 1)) & 0x55555555u;
+}
+
+// The query of a CTA where few coordinates settle early: every row of four consecutive coordinates per
+// lane, the first kF by a class of two bits in shared memory (bit 1: the cell counts below t, bit 0: above
+// -t; place n of a row at bits 2n, 2n + 1), the later ones from the table while a coordinate is undecided,
+// all cells for the full median of one that does not settle.
+template <int R>
+__device__ __forceinline__ void query_quads(const QueryParams& prm, const uint32_t* classes, uint32_t* sh, uint32_t pk) {
+  constexpr int kF = R / 2 + 1;
+  const uint32_t per_row = prm.c / 16;
+  const int64_t d = prm.d, nq = (d + 3) / 4;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t q0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); q0 < nq; q0 += stride) {
+    const int64_t q = q0 + (threadIdx.x & 31);
+    const int64_t i0 = q * 4;
+    const int tmax = q < nq ? (d - i0 < 4 ? (int)(d - i0) : 4) : 0;
+    float m[4] = {0.f, 0.f, 0.f, 0.f};
+    if (tmax > 0) {
+      float v[4][R];
+      uint32_t cell[4][kF];  // bucket of each of the first kF rows, sign bit of the cell in bit 31
+      uint32_t count[4] = {0u, 0u, 0u, 0u};  // cells below t in bits 0-7, above -t in bits 8-15
+      int lt[4], gt[4], rows[4];
+      bool done[4];
+#pragma unroll
+      for (int j = 0; j < kF; ++j) {
+        uint64_t x = affine61_nb(prm.h.a[j], prm.h.b[j], (uint32_t)i0);
+        uint64_t y = affine61_nb(prm.h.a2[j], prm.h.b2[j], (uint32_t)i0);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          cell[t][j] = 0u;
+          if (t < tmax) {
+            const uint32_t b = (uint32_t)x & prm.cmask, n = (b + 1u) & prm.cmask;
+            const uint32_t cls = (classes[j * per_row + (n >> 4)] >> ((n & 15u) * 2u)) & 3u;
+            // a negative sign swaps the two bits; one product puts each where it is counted
+            const uint32_t sg = (uint32_t)y & 1u;
+            count[t] += ((cls * (sg ? 0x81u : 0x201u)) >> (1u - sg)) & 0x101u;
+            cell[t][j] = b | signbit_of(y);
+            x = step61_nb(x, prm.h.a[j]);
+            y = step61_nb(y, prm.h.a2[j]);
+          }
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        lt[t] = (int)(count[t] & 0xFFu);
+        gt[t] = (int)(count[t] >> 8);
+        rows[t] = kF;
+        done[t] = pk != 0u && lt[t] >= kF && gt[t] >= kF;
+      }
+#pragma unroll
+      for (int j = kF; j < R; ++j) {
+        uint64_t x = affine61_nb(prm.h.a[j], prm.h.b[j], (uint32_t)i0);
+        uint64_t y = affine61_nb(prm.h.a2[j], prm.h.b2[j], (uint32_t)i0);
+        const float* row = prm.T + (size_t)j * prm.c;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          v[t][j] = 0.f;
+          if (t < tmax) {
+            if (!done[t]) {
+              v[t][j] = apply_sign(__ldg(row + ((uint32_t)x & prm.cmask)), signbit_of(y));
+              tally(v[t][j], pk, lt[t], gt[t]);
+              ++rows[t];
+            }
+            x = step61_nb(x, prm.h.a[j]);
+            y = step61_nb(y, prm.h.a2[j]);
+          }
+        }
+        if (j + 1 < R) {
+#pragma unroll
+          for (int t = 0; t < 4; ++t) done[t] = done[t] || (pk != 0u && lt[t] >= kF && gt[t] >= kF);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < kF; ++j) {
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          v[t][j] = 0.f;
+          if (t < tmax && !done[t])
+            v[t][j] = apply_sign(__ldg(prm.T + (size_t)j * prm.c + (cell[t][j] & 0x7FFFFFFFu)), cell[t][j] & 0x80000000u);
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        m[t] = done[t] ? __uint_as_float(pruned_marker(rows[t], rows[t] - kF)) : median_of<R>(v[t]);
+      store_est(prm, i0, tmax, m);
+    }
+#pragma unroll
+    for (int t = 0; t < 4; ++t) hist_add(sh, t < tmax ? (key_of(m[t]) >> kL1Shift) : kNone);
+  }
+}
+
 // HM: HEAVYMIX mode (prm.keys set): each coordinate's composite key is stored and histogrammed.
 template <int R, bool HM>
 __global__ void __launch_bounds__(kBitsBlock, 1) k_query_bits(const __grid_constant__ QueryParams prm,
@@ -741,25 +869,53 @@ __global__ void __launch_bounds__(kBitsBlock, 1) k_query_bits(const __grid_const
                                                               const __grid_constant__ GridSteps steps) {
   grid_begin();
   extern __shared__ uint4 sbits4[];
-  const uint32_t* sbits = reinterpret_cast<const uint32_t*>(sbits4);
+  uint32_t* sbits = reinterpret_cast<uint32_t*>(sbits4);
   __shared__ uint32_t sh[kBins];
   __shared__ uint32_t queues[kBitsBlock / 32][kQueue];
+  __shared__ uint32_t inside_cells;
   constexpr int kF = R / 2 + 1;
   constexpr bool kNextRow = kF + 1 < R;  // a marker names fewer than R rows
   const uint32_t per_row = prm.c / 32;
-  {
-    const int64_t n4 = (int64_t)kF * per_row * 2 / 4;
-    const uint4* src = reinterpret_cast<const uint4*>(words);
-    for (int64_t w = threadIdx.x; w < n4; w += blockDim.x) sbits4[w] = __ldcg(src + w);
-  }
+  const uint32_t half = kF * per_row;  // words of one kind of bit
   for (int b = threadIdx.x; b < kBins; b += blockDim.x) sh[b] = 0;
+  if (threadIdx.x == 0) inside_cells = 0;
   __syncthreads();
+  {
+    const uint4* src = reinterpret_cast<const uint4*>(words);
+    uint32_t n = 0;
+    for (uint32_t w = threadIdx.x; w < half / 2; w += blockDim.x) {
+      const uint4 x = __ldcg(src + w);
+      sbits4[w] = x;
+      n += (4 * w < half ? __popc(x.x) + __popc(x.y) : 0) + (4 * w + 2 < half ? __popc(x.z) + __popc(x.w) : 0);
+    }
+    n = __reduce_add_sync(kFull, n);
+    if ((threadIdx.x & 31) == 0 && n) atomicAdd(&inside_cells, n);
+  }
+  __syncthreads();
+  const uint32_t pk = prune_key_of(prm);
+  const double theta = HM ? __ldcg(prm.theta) : 0.0;
+  const float inside = (float)inside_cells / ((float)kF * (float)prm.c), open = left_open<R>(inside);
+  if (HM && prm.if_open && open > heavy_open(R)) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) prm.st->open = 1;
+    return;
+  }
+  if (!HM && open > kMostlyOpen && !(R >= 8 && inside < 0.3f && prm.c >= 1u << 14)) {
+    for (uint32_t w = threadIdx.x; w < half; w += blockDim.x) {
+      const uint32_t in = __ldcg(words + w), side = __ldcg(words + half + w);
+      const uint32_t below = in | side, above = in | ~side;
+      sbits[2 * w] = spread_bits(above) | spread_bits(below) << 1;
+      sbits[2 * w + 1] = spread_bits(above >> 16) | spread_bits(below >> 16) << 1;
+    }
+    __syncthreads();
+    query_quads<R>(prm, sbits, sh, pk);
+    hist_flush(sh, prm.hist, kBins);
+    last_block_pick(prm.hist, 11, prm.st, 0, prm.k);
+    return;
+  }
   const int64_t d = prm.d, nq = (d + 3) / 4;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int lane = threadIdx.x & 31;
   const uint32_t below = (1u << lane) - 1u;
-  const uint32_t pk = prune_key_of(prm);
-  const double theta = HM ? __ldcg(prm.theta) : 0.0;
   const float settled = __uint_as_float(pruned_marker(kF, 0));
   uint32_t* queue = queues[threadIdx.x >> 5];
   uint32_t n2 = 0, n3 = 0;  // entries in the queues, the same in every lane of the warp
@@ -1778,6 +1934,12 @@ int persistent_grid(K kernel, int64_t work_items, int block) {
 template <int R>
 cudaError_t launch_query_r(const QueryParams& p, cudaStream_t s) {
   auto kern = !is_pow2(p.c) ? k_query_mod<R> : p.keys ? k_query<R, true> : k_query<R, false>;
+  if (p.keys) {
+    // k_query_bits before it leaves an SM 28 KB of L1, in which few reads are in flight; a quarter of the SM's
+    // memory shared holds the resident CTAs' histograms (d = 25.6M, r = 5, c = 2^18, k = 4 c: 944 -> 568 us)
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 25);
+    if (e != cudaSuccess) return e;
+  }
   launch(kern, persistent_grid(kern, (p.d + 3) / 4, kBlock), kBlock, s, p);
   return cudaGetLastError();
 }
@@ -2004,6 +2166,7 @@ QueryParams make_query_params(const float* merged, const HashCoeffs& h, int r, u
   qp.vec = (reinterpret_cast<uintptr_t>(est) & 15u) == 0 ? 1 : 0;
   qp.pick = 1;
   qp.prune = 0;
+  qp.if_open = 0;
   qp.keys = nullptr;
   qp.theta = nullptr;
   qp.fill_seed = 0;
@@ -2236,8 +2399,16 @@ cudaError_t launch_query_heavymix(const float* merged, const HashCoeffs& h, int 
   qp.keys = keys;
   qp.theta = theta;
   qp.fill_seed = fill_seed;
-  if (prune && query_uses_bits(r, c)) err = launch_query_bits(qp, w, s);
-  else err = launch_query(qp, RowStrides(), s);
+  // The classified query first, where the classes fit; k_query where they do not, or where that query finds too
+  // few coordinates settled (its CTAs return at once otherwise).  Query with its selection in us, classified /
+  // k_query, d = 25.6M, r = 5, c = 2^18, k = 0.3 c, 0.6 c, c, 4 c: 239 / 454, 379 / 483, 483 / 491, 890 / 560.
+  // A row of squared norm l2sq has at most k cells that reach l2sq / k, and k / 0.76 that reach the bin edge
+  // below it: with k <= c / 8 five cells in six are inside, enough for any r, and k_query is not launched (the
+  // classified query then keeps the whole of it, also where the rows' norms differ widely).
+  const bool bits = prune && query_uses_bits(r, c);
+  qp.if_open = bits && k > (int64_t)c / 8 && heavy_open(r) < 1.f ? 1 : 0;
+  if (bits) err = launch_query_bits(qp, w, s);
+  if (err == cudaSuccess && (!bits || qp.if_open)) err = launch_query(qp, RowStrides(), s);
   if (err != cudaSuccess) return err;
   if ((err = mark(marks, 1, s)) != cudaSuccess) return err;
   const float* src = reinterpret_cast<const float*>(keys);
