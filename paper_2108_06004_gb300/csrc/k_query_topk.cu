@@ -2097,11 +2097,16 @@ constexpr WalkLauncher WalkTable<Rs...>::table[sizeof...(Rs)];
 // r/2 + 1 rows, so that two of them weigh more: r = 5, d = 25.6M, c = 2^20 395 / 342, r = 7, c = 2^18 510 / 444.
 constexpr int64_t kWalkQueryMinDim = int64_t(1) << 22;
 constexpr uint32_t kWalkQueryMinCols = 1u << 16;
+// With a large k few coordinates settle in the first rows and nearly all of them are queued, which a pruning walk
+// over a short vector does not repay: d = 4.2M, c = 2^18, k = d/30: r = 6 133 / 144, r = 8 177 / 197, r = 9 193 / 203
+// (d = 25.6M: within 3 % of each other).
+constexpr int64_t kWalkLargeKMinDim = int64_t(1) << 23;
 
 // The walk of a query, or false where k_query serves it.
 bool plan_walk(const QueryParams& p, const RowStrides& slow, WalkParams& wk) {
   if (slow.empty() || p.keys || p.r < (p.prune ? 3 : 5) || p.r > kWalkMaxRows || p.d < kWalkQueryMinDim || p.c < kWalkQueryMinCols)
     return false;
+  if (p.prune && p.d < kWalkLargeKMinDim && p.k > p.d / 200) return false;
   const int nr = p.prune ? p.r / 2 + 1 : p.r;
   const int64_t max_steps = p.d / ((int64_t)device_info().sms * 1024 * 2);
   PairShape best;
