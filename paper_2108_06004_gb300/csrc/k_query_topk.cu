@@ -1558,10 +1558,10 @@ __device__ __forceinline__ void for_keys(const float* __restrict__ src, int64_t 
   }
 }
 
-// picked: level 1 was picked already (st); otherwise it is picked from hist1 here, by every CTA.
+// hist1: the level-1 histogram of the keys; every CTA picks its bin here.
 __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThreads, 1)
     k_select_small(const float* __restrict__ src, int64_t d, int vec, uint32_t kmask, const uint32_t* __restrict__ hist1,
-                   const SelectState* st, int picked, uint32_t k, int64_t* __restrict__ idx_out) {
+                   uint32_t k, int64_t* __restrict__ idx_out) {
   grid_begin();
   extern __shared__ uint4 small_dyn[];
   SmallShared& sm = *reinterpret_cast<SmallShared*>(small_dyn);
@@ -1577,19 +1577,13 @@ __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThrea
 
   for (int b = threadIdx.x; b < kBins; b += kSmallThreads) {
     sm.h2[b] = 0;
-    sm.sum[b] = picked ? 0u : __ldcg(&hist1[b]);
+    sm.sum[b] = __ldcg(&hist1[b]);
   }
   for (int b = threadIdx.x; b < (1 << kL3Bits); b += kSmallThreads) sm.h3[b] = 0;
   for (int w = threadIdx.x; w < 2 * (int)per; w += kSmallThreads) gt_bm[w] = 0;  // both bitmaps
-  if (threadIdx.x == 0) {
-    sm.n = 0;
-    if (picked) {
-      sm.bin = __ldcg(&st->prefix);
-      sm.rem = __ldcg(&st->k_rem);
-    }
-  }
+  if (threadIdx.x == 0) sm.n = 0;
   __syncthreads();
-  if (!picked) pick_shared(sm, kBins, k);
+  pick_shared(sm, kBins, k);
   const uint32_t b1 = sm.bin, k1 = sm.rem;
   cluster.sync();  // every histogram is clear
 
@@ -2070,6 +2064,7 @@ constexpr ProbeLauncher ProbeTable<Rs...>::table[sizeof...(Rs)];
 // 2^22 coordinates up: below that the query takes a few tens of microseconds and the repair
 // kernel's launch costs more than the skipped rows save (measured on the 2^20 workload).
 constexpr int64_t kPruneMinDim = int64_t(1) << 22;
+static_assert(kPruneMinDim > kSmallMaxDim, "a pruning query needs the level-1 pick, which the cluster does by itself");
 bool can_prune(int r, uint32_t c, int64_t d) { return is_pow2(c) && r >= 3 && r <= GS_MAX_ROWS && d >= kPruneMinDim; }
 
 template <int R>
@@ -2290,9 +2285,8 @@ cudaError_t launch_query_bits(const QueryParams& p, const Workspace& w, cudaStre
   return T::table[p.r - 1](p, reinterpret_cast<uint32_t*>(w.cand), s);
 }
 
-// Levels 2 and 3 and the ordered output by one cluster; `picked`: see k_select_small.
-cudaError_t select_small(const float* src, int vec, uint32_t kmask, const uint32_t* hist1, const SelectState* st,
-                         int picked, int64_t d, int64_t k, int64_t* idx_out, cudaStream_t s) {
+// The selection by one cluster, from the level-1 histogram on.
+cudaError_t select_small(const float* src, int vec, uint32_t kmask, const uint32_t* hist1, int64_t d, int64_t k, int64_t* idx_out, cudaStream_t s) {
   cudaError_t e = cudaFuncSetAttribute(k_select_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_select_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)small_smem(kSmallMaxDim));
@@ -2307,7 +2301,7 @@ cudaError_t select_small(const float* src, int vec, uint32_t kmask, const uint32
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, k_select_small, src, d, vec, kmask, hist1, st, picked, (uint32_t)k, idx_out);
+  e = cudaLaunchKernelEx(&cfg, k_select_small, src, d, vec, kmask, hist1, (uint32_t)k, idx_out);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -2345,7 +2339,7 @@ cudaError_t launch_query_topk(const float* merged, const HashCoeffs& h, int r, u
   // rows are pruned only while the estimate stays internal: a caller's est_out gets every value
   const uint32_t j_target = sample_rank(d, k);
   qp.prune = (!est_out && can_prune(r, c, d) && j_target > 0) ? 1 : 0;
-  qp.pick = (qp.prune || !selects_small(d, k)) ? 1 : 0;  // k_repair needs the pick, and so do many CTAs
+  qp.pick = selects_small(d, k) ? 0 : 1;
   if (qp.prune) {
     using T = SampleTable<1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16>;
     if ((err = T::table[r - 1](qp, w.hist + 4 * kBins, j_target, s)) != cudaSuccess) return err;
@@ -2360,7 +2354,7 @@ cudaError_t launch_query_topk(const float* merged, const HashCoeffs& h, int r, u
     if ((err = T::table[r - 1](qp, w.hist + 3 * kBins, s)) != cudaSuccess) return err;
   }
   if ((err = mark(marks, 1, s)) != cudaSuccess) return err;
-  if (selects_small(d, k)) err = select_small(est, qp.vec, 0x7FFFFFFFu, w.hist, w.st, qp.pick, d, k, idx_out, s);
+  if (selects_small(d, k)) err = select_small(est, qp.vec, 0x7FFFFFFFu, w.hist, d, k, idx_out, s);
   else err = select_from_keys(w, est, qp.vec, 0x7FFFFFFFu, d, k, idx_out, s);
   return err != cudaSuccess ? err : mark(marks, 2, s);
 }
@@ -2400,7 +2394,7 @@ cudaError_t launch_query_heavymix(const float* merged, const HashCoeffs& h, int 
   // the query stores each coordinate's composite key and picks on their level-1 histogram
   QueryParams qp = make_query_params(merged, h, r, c, d, k, est, w.hist, w.st);
   qp.prune = prune;
-  qp.pick = (prune || !selects_small(d, k)) ? 1 : 0;
+  qp.pick = selects_small(d, k) ? 0 : 1;
   qp.keys = keys;
   qp.theta = theta;
   qp.fill_seed = fill_seed;
@@ -2417,7 +2411,7 @@ cudaError_t launch_query_heavymix(const float* merged, const HashCoeffs& h, int 
   if (err != cudaSuccess) return err;
   if ((err = mark(marks, 1, s)) != cudaSuccess) return err;
   const float* src = reinterpret_cast<const float*>(keys);
-  if (selects_small(d, k)) err = select_small(src, 1, 0xFFFFFFFFu, w.hist, w.st, qp.pick, d, k, idx_out, s);
+  if (selects_small(d, k)) err = select_small(src, 1, 0xFFFFFFFFu, w.hist, d, k, idx_out, s);
   else err = select_from_keys(w, src, 1, 0xFFFFFFFFu, d, k, idx_out, s);
   return err != cudaSuccess ? err : mark(marks, 2, s);
 }
@@ -2523,7 +2517,7 @@ cudaError_t launch_query_topk_noalloc(const float* merged, const HashCoeffs& h, 
   QueryParams qp = make_query_params(merged, h, r, c, d, k, est_out, hist, st);
   qp.pick = selects_small(d, k) ? 0 : 1;
   if ((err = launch_query(qp, slow, s)) != cudaSuccess) return err;
-  if (selects_small(d, k)) return select_small(est_out, qp.vec, 0x7FFFFFFFu, hist, st, 0, d, k, idx_out, s);
+  if (selects_small(d, k)) return select_small(est_out, qp.vec, 0x7FFFFFFFu, hist, d, k, idx_out, s);
   const int hgrid = persistent_grid(k_hist, (d + 3) / 4 / kU, kBlock);
   launch(k_hist, hgrid, kBlock, s, est_out, d, qp.vec, st, hist + kBins, kL2Shift, 11, 1);
   launch(k_hist, hgrid, kBlock, s, est_out, d, qp.vec, st, hist + 2 * kBins, 0, kL3Bits, 2);
