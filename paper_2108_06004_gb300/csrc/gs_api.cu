@@ -20,10 +20,12 @@ struct gs_sketch {
   float* tables;  // groups * r*c*W
   float* merged;  // r*c
   int device;
-  // c a power of two: the convergents of every row's rotation (chain_plan.h) by one coordinate and
-  // by a quad of four, else empty
-  std::vector<std::vector<gs::Convergent>> rotation, quad_rotation;
-  std::vector<std::vector<gs::Convergent>> slow;  // slow_strides of every row
+  // c a power of two: the convergents of every row's rotation (chain_plan.h), those of the first row's by a
+  // quad of four coordinates (its walk in the accumulate pass), and the slow strides of the first two rows
+  // (the query's walk); else empty
+  std::vector<std::vector<gs::Convergent>> rotation;
+  std::vector<gs::Convergent> quad_rotation;
+  std::vector<std::vector<gs::Convergent>> slow;
 };
 
 // Events recorded between the phases of a step while it is captured into a plan, where each
@@ -360,7 +362,7 @@ gs_status accumulate_insert_impl(gs_sketch* sk, int32_t first, int32_t n, float*
         // chains of at most 12 quads and one and a half waves of 768 threads per SM
         const int64_t nq = (d + 3) / 4, lanes = (int64_t)gs::device_info().sms * 768 * 3 / 2;
         const int64_t max_steps = std::min<int64_t>(12, std::max<int64_t>(1, nq * std::max(1, W / 4) / lanes));
-        const gs::ChainShape ch = gs::choose_chain(sk->quad_rotation[0], nq, kMinStride / 4, max_steps);
+        const gs::ChainShape ch = gs::choose_chain(sk->quad_rotation, nq, kMinStride / 4, max_steps);
         err = gs::launch_accumulate_chain(p, gs::QuadWalk{ch.stride, ch.steps, 0}, W, vec, s);
       } else {
         err = gs::launch_accumulate_insert(p, W, true, vec, s);
@@ -809,12 +811,11 @@ gs_status gs_sketch_create(int32_t r, int32_t c, uint64_t seed, int32_t workers,
   if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
   std::unique_ptr<gs_sketch> sk(new gs_sketch);
   derive_coefficients(r, seed, sk->h);
-  if (gs::is_pow2((uint32_t)c))
-    for (int j = 0; j < r; ++j) {
-      sk->rotation.push_back(gs::rotation_convergents(sk->h.a[j], (uint32_t)c));
-      sk->slow.push_back(gs::slow_strides(sk->rotation.back(), kMinStride));
-      sk->quad_rotation.push_back(gs::rotation_convergents(gs::mulmod61(4, sk->h.a[j]), (uint32_t)c));
-    }
+  if (gs::is_pow2((uint32_t)c)) {
+    for (int j = 0; j < r; ++j) sk->rotation.push_back(gs::rotation_convergents(sk->h.a[j], (uint32_t)c));
+    sk->quad_rotation = gs::rotation_convergents(gs::mulmod61(4, sk->h.a[0]), (uint32_t)c);
+    for (int j = 0; j < 2 && r >= 3; ++j) sk->slow.push_back(gs::slow_strides(sk->rotation[j], kMinStride));
+  }
   const int W = group_width ? group_width : choose_group_width(r, c, workers);
   const int groups = (workers + W - 1) / W;
   const size_t table_floats = (size_t)groups * r * c * W;

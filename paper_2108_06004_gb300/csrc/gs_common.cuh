@@ -297,7 +297,7 @@ cudaError_t launch_query_at(const float* T, const HashCoeffs& h, int r, uint32_t
 cudaError_t launch_add_sparse(float* T, const HashCoeffs& h, int r, uint32_t c, const int64_t* idx, const float* vals,
                               int64_t k, float scale, cudaStream_t s);
 cudaError_t launch_take(const float* src, int64_t n, const int64_t* idx, int64_t k, float* out, cudaStream_t s);
-// slow: the slow strides of every row (empty unless c is a power of two).
+// slow: the slow strides of the first two rows (empty unless c is a power of two and r >= 3).
 // marks (nullable): three events recorded, when set, before the query, between the query
 // (sample, median query, repair check) and the selection, and after the selection.
 cudaError_t launch_query_topk(const float* merged, const HashCoeffs& h, int r, uint32_t c,
