@@ -46,6 +46,7 @@ PER_CONFIG_STEPS = {"tiny-2^20": 300, "resnet18": 300, "resnet50": 100, "vgg16":
 PRUNE_MIN_DIM = 1 << 22  # the library skips query rows from this dimension on
 SAMPLE_PERIOD = 256      # ... with a prune-key sample of the first four of every 256 coordinates
 CLASS_BYTES = 192 << 10  # ... and classifies the first r/2 + 1 rows in shared memory when they fit
+WALK_MIN_COLS, WALK_MAX_ROWS = 1 << 16, 9  # ... else walks, where two rows share a walk
 
 
 def query_classifies(r: int, c: int) -> bool:
@@ -54,10 +55,27 @@ def query_classifies(r: int, c: int) -> bool:
     return 3 <= r <= 16 and c >= 64 and (c & (c - 1)) == 0 and (r // 2 + 1) * c // 4 <= CLASS_BYTES
 
 
+def query_kernels(r: int, c: int, d: int) -> tuple:
+    """(the kernels of the median query of a step, whether the markers count its requests).  A walk
+    keeps cells from one coordinate to the next, so that the cells which the markers name are not
+    reads; whether one serves the rows depends on their hash coefficients, which decides between the
+    two kernels named."""
+    pow2 = c & (c - 1) == 0
+    prunes = d >= PRUNE_MIN_DIM and r >= 3 and pow2
+    if prunes and query_classifies(r, c):
+        return f"k_qsample + k_pbits + k_query_bits<{r}> + k_repair", True
+    one = f"k_query<{r}>" if pow2 else f"k_query_mod<{r}>"
+    walks = pow2 and c >= WALK_MIN_COLS and 3 <= r <= WALK_MAX_ROWS and prunes
+    if walks:
+        one = f"k_query_walk<{r}> (or {one})"
+    return (f"k_qsample + {one} + k_repair" if prunes else one), not walks
+
 
 def insert_rows(W: int, r: int, c: int, d: int) -> int:
     """How many of the r rows (c a power of two) the accumulate pass of a group of W workers inserts;
-    the others go along chains of coordinates, which read the error vectors once more per row."""
+    the others go along chains of coordinates, which read the error vectors once more per row.  This is
+    what the library does with the workloads here; between 2^20 cell updates and 2^22 coordinates it
+    also weighs what the chains of a sketch's own coefficients save."""
     if d * r <= 1 << 20:
         return r
     if d < 1 << 22:
@@ -415,10 +433,11 @@ class Runner:
                 "gen": mean(per_step("gen")), "n": len(ins)}
 
     def query_rows(self):
-        """(fraction of coordinates that stopped early, rows examined per coordinate, table
-        cells read per coordinate) in the last query: a coordinate that stopped after examining
-        n rows, g of whose cells it read from the table, leaves -((32 g + n) * 2^-149) as its
-        estimate; every other coordinate read all r cells."""
+        """(fraction of coordinates that stopped early, rows examined per coordinate, cells taken
+        from the table per coordinate) in the last query: a coordinate that stopped after examining
+        n rows, g of whose cells were taken from the table, leaves -((32 g + n) * 2^-149) as its
+        estimate; every other coordinate took all r cells.  Along a walk a cell is taken once for many
+        coordinates, so that g says nothing of the reads."""
         import torch
         d, r = self.w.d, self.w.r
         bits = self.ws[: 4 * d].view(torch.int32)
@@ -447,7 +466,7 @@ def launches_per_step(run: Runner, variant: str) -> int:
     prunes = variant != "heavymix" and w.d >= PRUNE_MIN_DIM and w.r >= 3 and (w.c & (w.c - 1)) == 0
     inserts = run.groups * run.insert_launches
     bits = w.d >= PRUNE_MIN_DIM and query_classifies(w.r, w.c)
-    select = 1 if w.d <= 3 << 19 else 6               # one cluster up to 1.5 * 2^20 coordinates
+    select = 1 if w.d <= (25 << 15 if w.k > w.d // 100 else 3 << 19) else 6   # one cluster for short vectors
     if variant == "heavymix":
         # sumsq, theta, query (with the keys) + selection; k_query behind it where few may settle
         query = 3 + int(bits) + int(bits and w.k > w.c // 8 and w.r < 16) + select
@@ -560,24 +579,24 @@ def rooflines(run: Runner, variant: str, ph: dict, peaks, peak_kind, probes: dic
         prunes = d >= PRUNE_MIN_DIM and r >= 3 and (w.c & (w.c - 1)) == 0
         nq = (d + 3) // 4
         n_s = 4 * ((nq + SAMPLE_PERIOD // 4 - 1) // (SAMPLE_PERIOD // 4)) if prunes else 0
-        requests = d * cells_read + n_s * r
+        kernels, counted = query_kernels(r, w.c, d)
+        requests = d * cells_read + n_s * r if counted else None
         g_ms = probes.get("query_ms")
-        ach = requests / (q_ms / 1e3) / 1e9
+        ach = requests / (q_ms / 1e3) / 1e9 if counted else None
         q = {
-            "kernel": ((f"k_qsample + k_pbits + k_query_bits<{r}> + k_repair (median query, S4)"
-                        if query_classifies(r, w.c) else f"k_qsample + k_query_walk<{r}> + k_repair (median query, S4)")
-                       if prunes else f"k_query<{r}> (S4)") +
-                      (" and the S5 selection: eager, timed around the gs_query_topk call" if with_selection else ""),
+            "kernel": kernels + (" (median query, S4) and the S5 selection: eager, timed around the gs_query_topk call"
+                                 if with_selection else " (median query, S4)"),
             "bound": ("integer ALU pipe: the Mersenne hash of every row examined (the first rows' cells are "
                       "classified in shared memory, so few are read)" if prunes and query_classifies(r, w.c) else
                       "L1->L2 requests (scattered 4-byte reads of the merged table)"),
             "avg_ms": round(q_ms, 4), "pruned_fraction": round(pruned, 4), "rows_examined_per_coord": round(rows_read, 3),
-            "cells_read_per_coord": round(cells_read, 3),
-            "requests_per_step": requests, "requests_per_coord": round(requests / d, 3),
-            "achieved_G_requests_per_s": round(ach, 1),
+            "cells_read_per_coord": round(cells_read, 3) if counted else None,
+            "requests_per_step": requests, "requests_per_coord": round(requests / d, 3) if counted else None,
+            "achieved_G_requests_per_s": round(ach, 1) if counted else None,
             "peak_G_requests_per_s": None if g_ms is None else round(d * r / (g_ms / 1e3) / 1e9, 1),
             "peak_probe": "gs_query_request_ceiling: the query's loads of all r rows, no median or store",
-            "requests_frac_of_ceiling": None if g_ms is None else round(ach / (d * r / (g_ms / 1e3) / 1e9), 4),
+            "requests_frac_of_ceiling": (round(ach / (d * r / (g_ms / 1e3) / 1e9), 4)
+                                         if counted and g_ms is not None else None),
             "time_vs_full_read_ceiling": None if g_ms is None else round(g_ms / q_ms, 4),
             "hbm": {"algorithmic_bytes": 4 * d, "achieved_GBps": round(4 * d / (q_ms / 1e3) / 1e9, 1),
                     "frac": round(4 * d / (q_ms / 1e3) / 1e9 / peaks["hbm_gbs"], 4)},

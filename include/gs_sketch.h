@@ -176,9 +176,10 @@ gs_status gs_query_topk_workspace_size(int64_t d, int64_t k, size_t* bytes);
  * read are below a threshold t and at least f are above -t: then |est| < t whatever the
  * other rows hold, and it cannot be selected.  Its estimate is left in the workspace as the
  * marker -((32 g + n) * 2^-149): n the rows it examined (f <= n < r), g how many of those
- * cells were read from the table (where the classes of the first f rows' cells fit in shared
- * memory, f * c / 4 bytes <= 192 KiB, those cells are classified there and not read: g = n - f;
- * otherwise g = n).  The threshold is
+ * cells were taken from the table (where the classes of the first f rows' cells fit in shared
+ * memory, f * c / 4 bytes <= 192 KiB, those cells are classified there: g = n - f; otherwise
+ * g = n).  g is not a count of reads: where consecutive coordinates of a walk share a cell of
+ * the first two rows, it is read once for all of them.  The threshold is
  * taken by the same call before the main pass, from the full estimate of a fixed sample (the
  * first four coordinates of every 256): the level-1 bin edge below a rank of the sample chosen
  * so that the threshold lies under the k-th largest |est| except with negligible probability.
