@@ -19,7 +19,8 @@
 //                 the prune key skips its other rows and stores a marker (see below).  In its place:
 //                 k_query_bits (pruning, the first rows' cells classified in shared memory),
 //                 k_query_walk (long vectors, along a walk that keeps two rows' cells) and
-//                 k_query_mod (c not a power of two)
+//                 k_query_mod (c not a power of two); k_query_quads (HEAVYMIX: k_query) behind k_query_bits
+//                 takes the query over where few coordinates settle early
 //   k_repair      runs only if the level-1 pick fell below the prune key: recomputes every
 //                 marked estimate in full, rebuilds the level-1 histogram and picks again
 //   k_cand        one pass over est: keys above the picked level-1 bin are selected for
@@ -71,7 +72,7 @@ struct SelectState {
                        // query, before k_query, by k_qsample or k_heavy_theta
   uint32_t done_r;     // CTAs finished in k_repair
   uint32_t done_s;     // CTAs finished in k_qsample
-  uint32_t open;       // HEAVYMIX: k_query_bits left the whole query to k_query
+  uint32_t open;       // k_query_bits left the whole query to the kernel behind it
 };
 
 inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -248,8 +249,8 @@ struct QueryParams {
   int32_t vec;        // est 16-byte aligned
   int32_t pick;       // the last CTA picks the level-1 bin from the histogram of the keys
   int32_t prune;      // skip rows below st->prune_key (estimate internal to the workspace)
-  int32_t if_open;    // HEAVYMIX: k_query is launched behind k_query_bits and runs only where that kernel left the
-                      // query to it (st->open)
+  int32_t if_open;    // k_query_quads (HEAVYMIX: k_query) is launched behind k_query_bits and runs only where
+                      // that kernel left the query to it (st->open)
   uint32_t* keys;     // HEAVYMIX: also store each coordinate's composite key here, and build the
                       // level-1 histogram (and pick) on those keys instead of |est|
   const double* theta;  // HEAVYMIX: the threshold l2sq / k of H
@@ -663,8 +664,9 @@ __global__ void __launch_bounds__(kBlock, R <= 7 ? 3 : 2) k_query_walk(const __g
 //
 // The sorting pays while parts 1 and 2 settle enough coordinates; where most are left for part 3 (a large k,
 // many rows, few columns: the prune key lies within the cells' noise), evaluating every row of four
-// coordinates per lane from the start is the better order (query_quads), and a CTA takes it when the bits
-// say that more than kMostlyOpen of them will be left.  Query with its selection in us, sorted / quads,
+// coordinates per lane from the start is the better order (k_query_quads).  Every CTA takes the same sample of
+// the inside bits, and the query is left to that kernel, launched behind, where more than kMostlyOpen of the
+// coordinates would be left.  Query with its selection in us, sorted / quads,
 // d = 25.6M: r = 7, c = 2^16, k = d/1000, d/100, d/30, d/10 (shares left 0.19, 0.52, 0.71, 0.80) 277 / 440,
 // 456 / 478, 599 / 533, 652 / 551; r = 16, c = 2^14, k = d/1000 (0.97) 1450 / 1127.  The line is the one with the
 // least loss over 610 shapes (r 3 to 16, c 2^10 to 2^18, k d/10000 to d/3).  With many rows and few cells inside,
@@ -773,12 +775,29 @@ __device__ __forceinline__ uint32_t spread_bits(uint32_t x) {
   return (x | (x << 1)) & 0x55555555u;
 }
 
-// The query of a CTA where few coordinates settle early: every row of four consecutive coordinates per
+// The pruning query where few coordinates settle early: every row of four consecutive coordinates per
 // lane, the first kF by a class of two bits in shared memory (bit 1: the cell counts below t, bit 0: above
 // -t; place n of a row at bits 2n, 2n + 1), the later ones from the table while a coordinate is undecided,
-// all cells for the full median of one that does not settle.
+// all cells for the full median of one that does not settle.  A kernel of its own: within k_query_bits its
+// registers cost the sorted order 3 % (r = 5, d = 25.6M, c = 2^18: 186 -> 192 us).
 template <int R>
-__device__ __forceinline__ void query_quads(const QueryParams& prm, const uint32_t* classes, uint32_t* sh, uint32_t pk) {
+__global__ void __launch_bounds__(kBitsBlock, 1) k_query_quads(const __grid_constant__ QueryParams prm,
+                                                               const uint32_t* __restrict__ words) {
+  grid_begin();
+  if (__ldcg(&prm.st->open) == 0u) return;
+  extern __shared__ uint4 sbits4[];
+  uint32_t* classes = reinterpret_cast<uint32_t*>(sbits4);
+  __shared__ uint32_t sh[kBins];
+  const uint32_t half = (R / 2 + 1) * (prm.c / 32);  // words of one kind of bit
+  for (uint32_t w = threadIdx.x; w < half; w += blockDim.x) {
+    const uint32_t in = __ldcg(words + w), side = __ldcg(words + half + w);
+    const uint32_t below = in | side, above = in | ~side;
+    classes[2 * w] = spread_bits(above) | spread_bits(below) << 1;
+    classes[2 * w + 1] = spread_bits(above >> 16) | spread_bits(below >> 16) << 1;
+  }
+  for (int b = threadIdx.x; b < kBins; b += blockDim.x) sh[b] = 0;
+  __syncthreads();
+  const uint32_t pk = prune_key_of(prm);
   constexpr int kF = R / 2 + 1;
   const uint32_t per_row = prm.c / 16;
   const int64_t d = prm.d, nq = (d + 3) / 4;
@@ -860,6 +879,8 @@ __device__ __forceinline__ void query_quads(const QueryParams& prm, const uint32
 #pragma unroll
     for (int t = 0; t < 4; ++t) hist_add(sh, t < tmax ? (key_of(m[t]) >> kL1Shift) : kNone);
   }
+  hist_flush(sh, prm.hist, kBins);
+  last_block_pick(prm.hist, 11, prm.st, 0, prm.k);
 }
 
 // HM: HEAVYMIX mode (prm.keys set): each coordinate's composite key is stored and histogrammed.
@@ -869,47 +890,26 @@ __global__ void __launch_bounds__(kBitsBlock, 1) k_query_bits(const __grid_const
                                                               const __grid_constant__ GridSteps steps) {
   grid_begin();
   extern __shared__ uint4 sbits4[];
-  uint32_t* sbits = reinterpret_cast<uint32_t*>(sbits4);
+  const uint32_t* sbits = reinterpret_cast<const uint32_t*>(sbits4);
   __shared__ uint32_t sh[kBins];
   __shared__ uint32_t queues[kBitsBlock / 32][kQueue];
-  __shared__ uint32_t inside_cells;
   constexpr int kF = R / 2 + 1;
   constexpr bool kNextRow = kF + 1 < R;  // a marker names fewer than R rows
   const uint32_t per_row = prm.c / 32;
   const uint32_t half = kF * per_row;  // words of one kind of bit
-  for (int b = threadIdx.x; b < kBins; b += blockDim.x) sh[b] = 0;
-  if (threadIdx.x == 0) inside_cells = 0;
-  __syncthreads();
+  // one inside bit per thread, spread over the rows: a sample that every CTA takes alike
+  const uint32_t sampled = __ldcg(words + (uint32_t)((uint64_t)threadIdx.x * half / kBitsBlock));
   {
     const uint4* src = reinterpret_cast<const uint4*>(words);
-    uint32_t n = 0;
-    for (uint32_t w = threadIdx.x; w < half / 2; w += blockDim.x) {
-      const uint4 x = __ldcg(src + w);
-      sbits4[w] = x;
-      n += (4 * w < half ? __popc(x.x) + __popc(x.y) : 0) + (4 * w + 2 < half ? __popc(x.z) + __popc(x.w) : 0);
-    }
-    n = __reduce_add_sync(kFull, n);
-    if ((threadIdx.x & 31) == 0 && n) atomicAdd(&inside_cells, n);
+    for (uint32_t w = threadIdx.x; w < half / 2; w += blockDim.x) sbits4[w] = __ldcg(src + w);
   }
-  __syncthreads();
+  for (int b = threadIdx.x; b < kBins; b += blockDim.x) sh[b] = 0;
+  const float inside = (float)__syncthreads_count((sampled >> (threadIdx.x & 31)) & 1u) * (1.f / kBitsBlock);
   const uint32_t pk = prune_key_of(prm);
   const double theta = HM ? __ldcg(prm.theta) : 0.0;
-  const float inside = (float)inside_cells / ((float)kF * (float)prm.c), open = left_open<R>(inside);
-  if (HM && prm.if_open && open > heavy_open(R)) {
+  const float open = left_open<R>(inside);
+  if (prm.if_open && (HM ? open > heavy_open(R) : open > kMostlyOpen && !(R >= 8 && inside < 0.3f && prm.c >= 1u << 14))) {
     if (blockIdx.x == 0 && threadIdx.x == 0) prm.st->open = 1;
-    return;
-  }
-  if (!HM && open > kMostlyOpen && !(R >= 8 && inside < 0.3f && prm.c >= 1u << 14)) {
-    for (uint32_t w = threadIdx.x; w < half; w += blockDim.x) {
-      const uint32_t in = __ldcg(words + w), side = __ldcg(words + half + w);
-      const uint32_t below = in | side, above = in | ~side;
-      sbits[2 * w] = spread_bits(above) | spread_bits(below) << 1;
-      sbits[2 * w + 1] = spread_bits(above >> 16) | spread_bits(below >> 16) << 1;
-    }
-    __syncthreads();
-    query_quads<R>(prm, sbits, sh, pk);
-    hist_flush(sh, prm.hist, kBins);
-    last_block_pick(prm.hist, 11, prm.st, 0, prm.k);
     return;
   }
   const int64_t d = prm.d, nq = (d + 3) / 4;
@@ -1947,25 +1947,20 @@ struct QueryTable {
 template <int... Rs>
 constexpr QueryLauncher QueryTable<Rs...>::table[sizeof...(Rs)];
 
+int bits_grid(int64_t d) {
+  const int64_t need = ((d + 3) / 4 + kBitsBlock - 1) / kBitsBlock;
+  return (int)(need < device_info().sms ? (need < 1 ? 1 : need) : device_info().sms);
+}
+
 // k_query_bits<R> for a pruning query whose first rows' classes fit kBitsBytes: the classes are
 // written into `words` (f * c / 4 bytes of scratch) first.
-template <int R>
-cudaError_t launch_query_bits_r(const QueryParams& p, uint32_t* words, cudaStream_t s) {
-  constexpr int kF = R / 2 + 1;
-  const int64_t nwords = (int64_t)kF * (p.c / 32);  // words of one kind of bit
-  const int64_t warps = (nwords + kBlock / 32 - 1) / (kBlock / 32), cap = (int64_t)device_info().sms * 8;
-  launch(k_pbits, (int)(warps < cap ? warps : cap), kBlock, s, p.T, p.c, nwords, p.st, words);
-  auto kern = p.keys ? k_query_bits<R, true> : k_query_bits<R, false>;
-  const size_t smem = (size_t)nwords * 2 * sizeof(uint32_t);
+template <typename... KArgs, typename... Args>
+cudaError_t launch_on_every_sm(void (*kern)(KArgs...), int64_t d, size_t smem, cudaStream_t s, Args&&... args) {
   // the limit that every call sets: another thread's launch may stand between this call's setting and launch
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBitsBytes);
   if (e != cudaSuccess) return e;
-  const int64_t need = ((p.d + 3) / 4 + kBitsBlock - 1) / kBitsBlock;
-  const int grid = (int)(need < device_info().sms ? (need < 1 ? 1 : need) : device_info().sms);
-  GridSteps steps = {};
-  for (int j = 0; j < kF; ++j) steps.a[j] = 8 * mulmod61(p.h.a[j], (uint64_t)grid * kBitsBlock * 4);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
+  cfg.gridDim = dim3((unsigned)bits_grid(d));
   cfg.blockDim = dim3(kBitsBlock);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
@@ -1974,8 +1969,24 @@ cudaError_t launch_query_bits_r(const QueryParams& p, uint32_t* words, cudaStrea
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, kern, p, (const uint32_t*)words, steps);
+  e = cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
   return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <int R>
+cudaError_t launch_query_bits_r(const QueryParams& p, uint32_t* words, cudaStream_t s) {
+  constexpr int kF = R / 2 + 1;
+  const int64_t nwords = (int64_t)kF * (p.c / 32);  // words of one kind of bit
+  const int64_t warps = (nwords + kBlock / 32 - 1) / (kBlock / 32), cap = (int64_t)device_info().sms * 8;
+  launch(k_pbits, (int)(warps < cap ? warps : cap), kBlock, s, p.T, p.c, nwords, p.st, words);
+  const size_t smem = (size_t)nwords * 2 * sizeof(uint32_t);
+  GridSteps steps = {};
+  for (int j = 0; j < kF; ++j) steps.a[j] = 8 * mulmod61(p.h.a[j], (uint64_t)bits_grid(p.d) * kBitsBlock * 4);
+  auto kern = p.keys ? k_query_bits<R, true> : k_query_bits<R, false>;
+  cudaError_t e = launch_on_every_sm(kern, p.d, smem, s, p, (const uint32_t*)words, steps);
+  if (e == cudaSuccess && p.if_open && !p.keys)
+    e = launch_on_every_sm(k_query_quads<R>, p.d, smem, s, p, (const uint32_t*)words);
+  return e;
 }
 
 typedef cudaError_t (*BitsLauncher)(const QueryParams&, uint32_t*, cudaStream_t);
@@ -2278,6 +2289,24 @@ cudaError_t clear_selection(const Workspace& w, int64_t d, int64_t k, cudaStream
   return err;
 }
 
+// Whether k_query_quads is launched behind k_query_bits: were the cells noise alone, of standard deviation s, the
+// medians would deviate by 1.25 s / sqrt(r), their k-th largest would be the quantile of that, and the share p of
+// cells below it would follow.  Any structure in the vector raises the threshold and p; the prune key, a bin edge
+// below a sample's rank, lowers them (r = 7, k = d/100: 0.31 by this, 0.52 found), hence the margin of 0.3.  What is
+// not launched is not needed: k_query_bits then keeps the query whatever it finds.
+bool may_stay_open(int r, int64_t d, int64_t k) {
+  const double tail = (double)k / (double)d;
+  double lo = 0.0, hi = 8.0;  // erfc(z) = tail
+  for (int n = 0; n < 24; ++n) {
+    const double z = 0.5 * (lo + hi);
+    (std::erfc(z) > tail ? lo : hi) = z;
+  }
+  const double p = std::erf(lo * 1.2533 / std::sqrt((double)r));
+  const int f = r / 2 + 1;
+  const double few = std::pow(p, f - 1);
+  return 1.0 - few * p - (f + 1 < r ? f * few * (1.0 - p) * p : 0.0) > kMostlyOpen - 0.3;
+}
+
 // The pruning query by k_query_bits; its words go in the candidate area, which the selection only
 // uses after the query.
 cudaError_t launch_query_bits(const QueryParams& p, const Workspace& w, cudaStream_t s) {
@@ -2345,6 +2374,7 @@ cudaError_t launch_query_topk(const float* merged, const HashCoeffs& h, int r, u
     if ((err = T::table[r - 1](qp, w.hist + 4 * kBins, j_target, s)) != cudaSuccess) return err;
   }
   if (qp.prune && query_uses_bits(r, c)) {
+    qp.if_open = may_stay_open(r, d, k) ? 1 : 0;
     if ((err = launch_query_bits(qp, w, s)) != cudaSuccess) return err;
   } else if ((err = launch_query(qp, slow, s)) != cudaSuccess) {
     return err;

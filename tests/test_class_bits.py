@@ -67,7 +67,7 @@ def _spread(x):
 
 
 def test_classes_from_bits():
-    """query_quads' classes: two bits per place out of the inside and side words, which a coordinate's sign
+    """k_query_quads' classes: two bits per place out of the inside and side words, which a coordinate's sign
     swaps and one product adds to the packed counters."""
     rng = np.random.default_rng(7)
     for _ in range(200):
