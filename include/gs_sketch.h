@@ -83,7 +83,7 @@ gs_status gs_sketch_destroy(gs_sketch* sketch);
 
 /* Shape query: any output pointer may be NULL.  rows_per_pass is the number of rows the fused
  * insert updates per pass over the vectors when it sends one reduction per coordinate and row (c
- * not a power of two, or gradients read from host memory). */
+ * not a power of two, gradients read from host memory, or rows whose chains would save too few). */
 gs_status gs_sketch_info(const gs_sketch* sketch, int32_t* r, int32_t* c, int32_t* workers,
                          int32_t* group_width, int32_t* rows_per_pass);
 

@@ -123,12 +123,15 @@ __device__ __forceinline__ void red_add_v4(float* p, float v0, float v1, float v
 }
 
 // ---- L2 eviction priorities -------------------------------------------------------------
-// Cache policies for the insert: the sketch table receives every reduction and should stay in L2
-// (evict_last).  Vector streams are marked evict_first only where the table does not fit L2 beside
-// them (64 MiB row slices and 8 workers' streams: five row passes 21.9 ms with both policies, 25.0
-// without).  Elsewhere evict_first costs: a line that two warps share, as every line of a vector
-// that does not start on a 128-byte boundary does, may be evicted half written.  Accumulating 8
-// vectors of 25,557,032, 32 bytes off such a boundary: 0.645 ms without the mark, 0.745 with it.
+// Cache policies for the insert.  The sketch table receives every reduction and should stay in L2:
+// evict_last in every kernel.  Vector streams: normal in k_accumulate_chain; in k_insert_chain, which
+// only reads them, evict_first once the vectors no longer fit L2 from one row to the next
+// (ChainParams::resident); in the insert by reductions evict_first only where the table needs several
+// passes (InsertParams::evict; 64 MiB row slices and 8 workers' streams, every row by reductions: five row
+// passes 21.9 ms with both policies, 25.0 without).  Streams that are written must not carry it lightly: a
+// line that two warps share, as every line of a vector that does not start on a 128-byte boundary does, may
+// be evicted half written.  Accumulating 8 vectors of 25,557,032, 32 bytes off such a boundary: 0.645 ms
+// without the mark, 0.745 with it.
 __device__ __forceinline__ uint64_t policy_evict_first() {
   uint64_t pol;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));

@@ -19,7 +19,8 @@
 //
 // For c a power of two the buckets of a row form a rotation, and a row can be inserted along
 // chains of coordinates that share a bucket (chain_plan.h): k_insert_chain needs one reduction for
-// about ten coordinates, at the price of reading the vectors once more for the row.
+// about ten coordinates, at the price of reading the vectors once more for the row.  Which rows go which
+// way is decided in gs_api.cu.
 #include "gs_common.cuh"
 
 namespace gs {
@@ -231,11 +232,12 @@ __global__ void __launch_bounds__(kBlock) k_accumulate_insert_coop(const __grid_
 // The accumulate pass along chains of quads (c a power of two): row prm.j0 keeps its buckets along a
 // chain, so its values are summed in registers and its cells updated only when a bucket changes;
 // rows prm.j0 + 1 .. prm.j1 - 1 take one reduction per coordinate as above.  Every lane holds one
-// quad of min(W, 4) workers.  At W = 8 the pass is bound by HBM with up to three such rows
-// (0.72, 0.75, 0.83 ms for 1, 2, 3 rows of 8 workers at d = 25,557,032; 0.94 and 1.08 ms for 4 and
-// 5, where the reductions take over).  Loads go through L1, where neighbouring warps find the rest
-// of the lines they share when a vector does not start on a 128-byte boundary: the times are the
-// same for both, while k_accumulate_insert_coop takes 0.83 ms for three rows of aligned vectors and
+// quad of min(W, 4) workers.  The path through L1TEX bounds it, which the reductions share with the
+// streams: 8 workers, d = 25,557,032: 0.72, 0.75, 0.83 ms for 1, 2, 3 rows (84 % of the measured copy rate with
+// one), 0.94 and 1.08 for 4 and 5; with four rows L1TEX is busy 84 % of the time and DRAM 55 %.  With one
+// row DRAM reaches 74 % at 36 % of the warps (72 registers).  Loads go through L1, where neighbouring
+// warps find the rest of the lines they share when a vector does not start on a 128-byte boundary: the
+// times are the same for both, while k_accumulate_insert_coop takes 0.83 ms for three rows of aligned vectors and
 // 0.95 ms off the boundary.  Staging the next step in shared memory by cp.async was slower (0.88 ms
 // for one row): it halves the resident warps.
 template <int N>
